@@ -298,8 +298,9 @@ void sweep_graph_destroy(void* graph);
  * number of launches.  Cost: two event records per recorded launch, and an
  * event between two kernels ends their programmatic overlap. */
 enum {
-  SWEEP_K_AC_FWD = 0,     /* acoustic forward step (all its kernels)   */
-  SWEEP_K_AC_BWD = 1,     /* acoustic backward step (all its kernels)  */
+  SWEEP_K_AC_FWD = 0,     /* acoustic forward step (all its kernels; on
+                             small problems one launch carries up to 3)  */
+  SWEEP_K_AC_BWD = 1,     /* acoustic backward step (the same)         */
   SWEEP_K_EL_VEL = 2,     /* elastic velocity half step                */
   SWEEP_K_EL_STR = 3,     /* elastic stress step                       */
   SWEEP_K_AC_FWD_IN = 4,  /* acoustic forward, stencil kernel          */

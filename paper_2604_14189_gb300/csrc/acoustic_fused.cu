@@ -1,0 +1,121 @@
+// Fused acoustic kernels (see acoustic_fused.cuh): the launch variants and
+// the rule that chooses one of them, or the per-step stencil + CPML kernels,
+// for a problem.
+#include <algorithm>
+
+#include "acoustic_fused.cuh"
+
+namespace sweep {
+namespace {
+
+template <class C, int RES>
+__global__ void __launch_bounds__(C::NT, RES)
+    ac_fused_fwd_kernel(const __grid_constant__ AcFusedArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  FusedFwdSmem<C>& m = *reinterpret_cast<FusedFwdSmem<C>*>(smem_raw);
+  fused_fwd_body<C>(a, m, reinterpret_cast<int2*>(&m + 1));
+}
+
+template <class C, int RES>
+__global__ void __launch_bounds__(C::NT, RES)
+    ac_fused_bwd_kernel(const __grid_constant__ AcFusedArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  FusedBwdSmem<C>& m = *reinterpret_cast<FusedBwdSmem<C>*>(smem_raw);
+  int2* list = reinterpret_cast<int2*>(&m + 1);
+  fused_bwd_body<C>(a, m, list, reinterpret_cast<float*>(list + (a.res ? a.g.nrec : 0)));
+}
+
+struct Variant {
+  FusedShape s;
+  int res, waves;          // CTAs per SM; most waves it is used for
+  int threads;
+  size_t smem, rec_bytes;  // fixed shared memory, and more per receiver
+  void (*kernel)(const AcFusedArgs);
+};
+
+template <int T, int BZ, int BX, int V, int RES, int WAVES>
+Variant fwd_variant() {
+  using C = FusedTile<T, BZ, BX, V>;
+  return {{T, BZ, BX}, RES, WAVES, C::NT, sizeof(FusedFwdSmem<C>), sizeof(int2),
+          ac_fused_fwd_kernel<C, RES>};
+}
+template <int T, int BZ, int BX, int V, int RES, int WAVES>
+Variant bwd_variant() {
+  using C = FusedTile<T, BZ, BX, V>;
+  return {{T, BZ, BX}, RES, WAVES, C::NT, sizeof(FusedBwdSmem<C>), sizeof(int2) + 4 * T,
+          ac_fused_bwd_kernel<C, RES>};
+}
+
+// Fastest first.  A launch costs about the same however few of its CTAs'
+// slots are used, so the variant with the most steps per launch whose CTAs
+// still run at once is the fastest: us per step on GB300 (200 x 200 + 40
+// grids of 1, 2, 3, 4, 6, 8 shots; the 141 x 187 + 23 grid of 3 for the second
+// variants) against the stencil + CPML kernels' 4.4, 4.5, 4.6, 5.1, 6.3, 7.1
+// forward and 8.7, 8.6, 8.7, 9.0, 9.7, 13.0 backward (with illumination):
+//   forward   3 steps, 24 x 24, one CTA per SM: 1.9 | 3.4 | 4.7 | 6.0 | 8.5
+//             2 steps, 32 x 32, one: 2.3 (141 x 187)
+//             2 steps, 24 x 24, two: 2.5 | 2.5 | 3.7 | 4.2 | 5.9
+//             2 steps, 24 x 24, three: 3.1 | 3.1 | 3.2 | 4.5 | 5.3 | 6.8
+//   backward  2 steps, 24 x 24, one: 4.0 | 6.5 | 8.7
+//             2 steps, 32 x 32, one: 5.0 (141 x 187)
+//             1 step, 16 x 32, three: 5.8 | 5.7 | 8.6 | 9.3
+//             1 step, 32 x 32, two: 6.6 | 6.8 | 6.6 | 9.6
+// Past one wave (forward: two of the last variant) the per-step kernels,
+// which pipeline their loads, are faster: 301 x 901 + 40 with 20 shots takes
+// them 26.6 us forward against 61.  Whole calls: 200 x 200 + 40 forward, 1000
+// steps, 4.40 -> 1.91 ms; 141 x 187 + 23 gradient, 3 shots, 900 steps, 10.8 ->
+// 6.0 ms.
+const Variant* variants(int dir, int* n) {
+  static const Variant f[] = {fwd_variant<3, 24, 24, 4, 1, 1>(), fwd_variant<2, 32, 32, 4, 1, 1>(),
+                              fwd_variant<2, 24, 24, 4, 2, 1>(), fwd_variant<2, 24, 24, 4, 3, 2>()};
+  static const Variant b[] = {bwd_variant<2, 24, 24, 2, 1, 1>(), bwd_variant<2, 32, 32, 4, 1, 1>(),
+                              bwd_variant<1, 16, 32, 4, 3, 1>(), bwd_variant<1, 32, 32, 4, 2, 1>()};
+  *n = dir ? (int)(sizeof(b) / sizeof(b[0])) : (int)(sizeof(f) / sizeof(f[0]));
+  return dir ? b : f;
+}
+
+constexpr size_t kMaxSmem = 227 * 1024;
+
+}  // namespace
+
+int fused_variant(const Geom& g, int dir) {
+  if (g.nrec > kFusedMaxRec || g.nshot < 1) return -1;
+  int n;
+  const Variant* v = variants(dir, &n);
+  const long long sms = device_sms();
+  for (int i = 0; i < n; ++i) {
+    const long long ctas = (long long)((g.NX + v[i].s.bx - 1) / v[i].s.bx) *
+                           ((g.NZ + v[i].s.bz - 1) / v[i].s.bz) * g.nshot;
+    if (ctas <= sms * v[i].res * v[i].waves) return i;
+  }
+  return -1;
+}
+
+FusedShape fused_shape(int dir, int v) {
+  int n;
+  return variants(dir, &n)[v].s;
+}
+
+void launch_ac_fused(int dir, int v, const AcFusedArgs& a, cudaStream_t st) {
+  int n;
+  const Variant& V = variants(dir, &n)[v];
+  static const bool attr = [] {  // thread-safe one-time initialisation
+    for (int d = 0; d < 2; ++d) {
+      int k;
+      const Variant* all = variants(d, &k);
+      for (int i = 0; i < k; ++i)
+        cudaFuncSetAttribute(all[i].kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)std::min(all[i].smem + all[i].rec_bytes * kFusedMaxRec, kMaxSmem));
+    }
+    return true;
+  }();
+  (void)attr;
+  const Geom& g = a.g;
+  const bool rec = dir ? a.res != nullptr : a.data != nullptr;
+  const dim3 grid((g.NX + V.s.bx - 1) / V.s.bx, (g.NZ + V.s.bz - 1) / V.s.bz, g.nshot);
+  launch_dependent(V.kernel, grid, dim3(V.threads), V.smem + (rec ? V.rec_bytes * g.nrec : 0),
+                   st, a);
+  note_launches(1);
+}
+
+}  // namespace sweep

@@ -112,6 +112,8 @@ struct Layout {
   size_t status = 0, partial = 0, vmax = 0, K = 0;
   size_t ax = 0, bx = 0, az = 0, bz = 0, axh = 0, bxh = 0, azh = 0, bzh = 0;
   size_t u[2] = {0, 0}, psx[2] = {0, 0}, psz[2] = {0, 0}, zex = 0, zez = 0;
+  // fused kernels: the second set of the state (u and mu pairs, zeta)
+  size_t u2[2] = {0, 0}, m2[2] = {0, 0}, zex2 = 0, zez2 = 0;
   size_t m[2] = {0, 0}, pbx[2] = {0, 0}, pbz[2] = {0, 0}, zbx[2] = {0, 0}, zbz[2] = {0, 0};
   size_t data = 0, save = 0, graw = 0, iraw = 0;
   size_t el_par[5] = {0, 0, 0, 0, 0};  // elastic coefficients
@@ -183,6 +185,19 @@ bool valid_problem(const sweep_problem* p) {
   const long long tiles = (NZ + 15) / 16 * ((NX + 127) / 128);  // smallest tiles in use
   if (tiles * p->nshot >= (1LL << 31)) return false;
   return true;
+}
+
+// Deterministic mode of a problem: one writer per border cell and phase.
+bool deterministic(const sweep_problem* p) {
+  return (p->flags & SWEEP_F_DETERMINISTIC) != 0;
+}
+
+// The fused kernels' variant for a problem's forward (dir 0) or backward
+// (dir 1) loop; -1: the stencil and CPML kernels.
+int fused_of(const sweep_problem* p, int dir) {
+  if (p->physics != SWEEP_ACOUSTIC || deterministic(p) || (p->flags & SWEEP_F_ONE_LAUNCH))
+    return -1;
+  return fused_variant(make_geom(p), dir);
 }
 
 Layout layout(const sweep_problem* p, int mode) {
@@ -271,6 +286,16 @@ Layout layout(const sweep_problem* p, int mode) {
     L.graw = b.take(F);
     L.iraw = b.take(F);
   }
+  const bool ff = mode != SWEEP_MODE_ADJOINT && fused_of(p, 0) >= 0;
+  const bool fb = mode != SWEEP_MODE_FORWARD && fused_of(p, 1) >= 0;
+  if (ff || (fb && mode == SWEEP_MODE_GRADIENT))
+    for (size_t& o : L.u2) o = b.take(F);
+  if (ff) {  // a gradient's backward buffers are free during its forward loop
+    L.zex2 = mode == SWEEP_MODE_GRADIENT ? L.zbx[0] : b.take(F);
+    L.zez2 = mode == SWEEP_MODE_GRADIENT ? L.zbz[0] : b.take(F);
+  }
+  if (fb)  // and psi is free during its backward loop
+    for (int i = 0; i < 2; ++i) L.m2[i] = mode == SWEEP_MODE_GRADIENT ? L.psx[i] : b.take(F);
   L.total = b.off;
   return L;
 }
@@ -344,11 +369,6 @@ bool z_map(const Geom& g, const float* base, CUtensorMap* m, int rows) {
 // The shared K grid [NZ][NXp] with box (bx, bz).
 bool map2(CUtensorMap* m, const Geom& g, const float* base, uint32_t bx, uint32_t bz) {
   return make_tensor_map(m, base, 2, g.NX, g.NZ, 1, g.NXp, (uint64_t)g.fstride, bx, bz, 1);
-}
-
-// Deterministic mode of a problem: one writer per border cell and phase.
-bool deterministic(const sweep_problem* p) {
-  return (p->flags & SWEEP_F_DETERMINISTIC) != 0;
 }
 
 // Rows of the acoustic stencil tiles of a problem.
@@ -444,9 +464,79 @@ struct AcFwdLoop {
   }
 };
 
+// The arguments that every launch of a fused loop shares.
+AcFusedArgs fused_args(const sweep_problem* p, const Layout& L, void* ws, const float* wavelet,
+                       const int32_t* src, const int32_t* rec) {
+  AcFusedArgs a{};
+  a.g = make_geom(p);
+  a.K = at<float>(ws, L.K);
+  a.ax = at<float>(ws, L.ax);
+  a.bx = at<float>(ws, L.bx);
+  a.az = at<float>(ws, L.az);
+  a.bz = at<float>(ws, L.bz);
+  a.wavelet = wavelet;
+  a.src = src;
+  a.rec = rec;
+  a.status = at<int>(ws, L.status);
+  return a;
+}
+
+// Forward loop through the fused kernels: launch k reads state set k % 2 and
+// writes the other one.  The sets are named so that u^{nt} ends in u[nt % 2]
+// and u^{nt-1} in the other, as acoustic_forward_loop leaves them.
+int fused_forward_loop(const sweep_problem* p, const Layout& L, void* ws, int variant,
+                       const float* wavelet, const int32_t* src, const int32_t* rec, float* data,
+                       bool save_ring, cudaStream_t st) {
+  PhaseRange r("sweep acoustic forward");
+  AcFusedArgs a = fused_args(p, L, ws, wavelet, src, rec);
+  const Geom& g = a.g;
+  const size_t F = sizeof(float) * (size_t)g.fstride * (size_t)g.nshot;
+  cudaMemsetAsync(at<char>(ws, L.fwd_lo), 0, L.fwd_hi - L.fwd_lo, st);
+  cudaMemsetAsync(at<char>(ws, L.zex2), 0, F, st);
+  cudaMemsetAsync(at<char>(ws, L.zez2), 0, F, st);
+  a.data = g.nrec > 0 ? data : nullptr;
+  a.save = save_ring ? at<float>(ws, L.save) : nullptr;
+  const int T = fused_shape(0, variant).T;
+  const int last = (g.nt + T - 1) / T % 2, A = g.nt & 1;
+  size_t u[2], up[2];
+  u[last] = L.u[A];
+  up[last] = L.u[A ^ 1];
+  u[last ^ 1] = L.u2[0];
+  up[last ^ 1] = L.u2[1];
+  if (last == 1)  // u^0 and u^{-1}
+    for (size_t o : L.u2) cudaMemsetAsync(at<char>(ws, o), 0, F, st);
+  const size_t zx[2] = {L.zex, L.zex2}, zz[2] = {L.zez, L.zez2};
+  void* loop = profile_begin(SWEEP_K_AC_FWD_LOOP, st);
+  int k = 0;
+  for (int n = 0; n < g.nt; n += T, ++k) {
+    const int i = k & 1, o = i ^ 1;
+    a.n = n;
+    a.steps = std::min(T, g.nt - n);
+    a.ui = at<float>(ws, u[i]);
+    a.upi = at<float>(ws, up[i]);
+    a.pzi = at<float>(ws, L.psz[i]);
+    a.pxi = at<float>(ws, L.psx[i]);
+    a.zzi = at<float>(ws, zz[i]);
+    a.zxi = at<float>(ws, zx[i]);
+    a.uo = at<float>(ws, u[o]);
+    a.upo = at<float>(ws, up[o]);
+    a.pzo = at<float>(ws, L.psz[o]);
+    a.pxo = at<float>(ws, L.psx[o]);
+    a.zzo = at<float>(ws, zz[o]);
+    a.zxo = at<float>(ws, zx[o]);
+    void* tok = profile_begin(SWEEP_K_AC_FWD, st);
+    launch_ac_fused(0, variant, a, st);
+    profile_end(tok, st);
+  }
+  profile_end(loop, st);
+  return SWEEP_OK;
+}
+
 int acoustic_forward_loop(const sweep_problem* p, const Layout& L, void* ws,
                           const float* wavelet, const int32_t* src, const int32_t* rec,
                           float* data, bool save_ring, cudaStream_t st) {
+  if (const int v = fused_of(p, 0); v >= 0)
+    return fused_forward_loop(p, L, ws, v, wavelet, src, rec, data, save_ring, st);
   PhaseRange r("sweep acoustic forward");
   AcFwdLoop f;
   const int rc = f.init(p, L, ws, wavelet, src, rec, data, save_ring, st);
@@ -581,10 +671,75 @@ struct AcBwdLoop {
   }
 };
 
+// Backward loop through the fused kernels, from (u^{nt-1}, u^{nt}) as either
+// forward loop leaves them.
+int fused_backward_loop(const sweep_problem* p, const Layout& L, void* ws, int variant,
+                        const float* wavelet, const int32_t* src, const int32_t* rec,
+                        const float* res, float* wgrad, bool imaging, bool illum,
+                        cudaStream_t st) {
+  PhaseRange r("sweep acoustic backward");
+  AcFusedArgs a = fused_args(p, L, ws, wavelet, src, rec);
+  const Geom& g = a.g;
+  const size_t F = sizeof(float) * (size_t)g.fstride * (size_t)g.nshot;
+  cudaMemsetAsync(at<char>(ws, L.adj_lo), 0, L.adj_hi - L.adj_lo, st);
+  const int T = fused_shape(1, variant).T;
+  size_t u[2] = {0, 0}, up[2] = {0, 0};
+  if (imaging) {
+    cudaMemsetAsync(at<float>(ws, L.graw), 0, F, st);
+    if (illum) cudaMemsetAsync(at<float>(ws, L.iraw), 0, F, st);
+    const int A = g.nt & 1;
+    u[0] = L.u[A ^ 1];  // u^{nt-1}
+    up[0] = L.u[A];
+    u[1] = L.u2[0];
+    up[1] = L.u2[1];
+    a.save = at<float>(ws, L.save);
+    a.graw = at<float>(ws, L.graw);
+    a.illum = illum ? at<float>(ws, L.iraw) : nullptr;
+  }
+  a.imaging = imaging;
+  a.res = g.nrec > 0 ? res : nullptr;
+  a.wgrad = wgrad;
+  const size_t m[2] = {L.m[0], L.m2[0]}, mp[2] = {L.m[1], L.m2[1]};
+  void* loop = profile_begin(SWEEP_K_AC_BWD_LOOP, st);
+  // step 0 only images and gathers the wavelet adjoint
+  const int last = imaging || wgrad ? 0 : 1;
+  int k = 0;
+  for (int n = g.nt; n >= last; n -= T, ++k) {
+    const int i = k & 1, o = i ^ 1;
+    a.n = n;
+    a.steps = std::min(T, n - last + 1);
+    a.mi = at<float>(ws, m[i]);
+    a.mpi = at<float>(ws, mp[i]);
+    a.pzi = at<float>(ws, L.pbz[i]);
+    a.pxi = at<float>(ws, L.pbx[i]);
+    a.zzi = at<float>(ws, L.zbz[i]);
+    a.zxi = at<float>(ws, L.zbx[i]);
+    if (imaging) {
+      a.ui = at<float>(ws, u[i]);
+      a.upi = at<float>(ws, up[i]);
+      a.uo = at<float>(ws, u[o]);
+      a.upo = at<float>(ws, up[o]);
+    }
+    a.mo = at<float>(ws, m[o]);
+    a.mpo = at<float>(ws, mp[o]);
+    a.pzo = at<float>(ws, L.pbz[o]);
+    a.pxo = at<float>(ws, L.pbx[o]);
+    a.zzo = at<float>(ws, L.zbz[o]);
+    a.zxo = at<float>(ws, L.zbx[o]);
+    void* tok = profile_begin(SWEEP_K_AC_BWD, st);
+    launch_ac_fused(1, variant, a, st);
+    profile_end(tok, st);
+  }
+  profile_end(loop, st);
+  return SWEEP_OK;
+}
+
 int acoustic_backward_loop(const sweep_problem* p, const Layout& L, void* ws,
                            const float* wavelet, const int32_t* src, const int32_t* rec,
                            const float* res, float* wgrad, bool imaging, bool illum,
                            cudaStream_t st) {
+  if (const int v = fused_of(p, 1); v >= 0)
+    return fused_backward_loop(p, L, ws, v, wavelet, src, rec, res, wgrad, imaging, illum, st);
   PhaseRange r("sweep acoustic backward");
   AcBwdLoop b;
   const int rc = b.init(p, L, ws, wavelet, src, rec, res, wgrad, imaging, illum, st);

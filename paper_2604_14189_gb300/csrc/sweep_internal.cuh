@@ -225,6 +225,40 @@ int launch_ac_loop_bwd(const LoopArgs& a, cudaStream_t st);
 // latches SWEEP_ETIMEOUT in *status; bar: 4 words of scratch.
 int launch_barrier_timeout_check(unsigned* bar, int* status, cudaStream_t st);
 
+// Fused kernels (acoustic_fused.cu): one launch takes up to T steps of every
+// (tile, shot).  A variant fixes T and the tile; the state is read from one
+// set of buffers and written to another (neighbouring tiles read halos of the
+// former).  Forward: steps n, n + 1, ... from (u^n, u^{n-1}); backward: steps
+// n, n - 1, ... from (mu^{n+1}, mu^{n+2}) and, with imaging, (u^n, u^{n+1})
+// ((u^{nt-1}, u^{nt}) for n = nt, whose step leaves u alone).
+struct AcFusedArgs {
+  Geom g;
+  const float *K, *ax, *bx, *az, *bz;
+  // in: u^n and u^{n-1} (u^{n+1} backward), mu^{n+1} and mu^{n+2}, the memory
+  // variables (psi, zeta or their adjoints) per axis; out: the same after
+  // the launch
+  const float *ui, *upi, *mi, *mpi, *pzi, *zzi, *pxi, *zxi;
+  float *uo, *upo, *mo, *mpo, *pzo, *zzo, *pxo, *zxo;
+  const float* wavelet;
+  const int32_t *src, *rec;
+  float* data;       // forward: traces or null
+  const float* res;  // backward: residual [S][nrec][nt] or null
+  float* save;       // ring slot of u^0 or null
+  float *graw, *illum, *wgrad;  // backward; illum, wgrad or null
+  int* status;
+  int n, steps;      // first step, steps of this launch (<= T)
+  int imaging;
+};
+struct FusedShape {
+  int T, bz, bx;  // steps per launch, tile rows and columns
+};
+constexpr int kFusedMaxRec = 2048;  // receivers per shot a CTA can list
+// The variant a problem's forward (dir 0) or backward (dir 1) loop runs, or
+// -1: the stencil + CPML kernels are the faster ones.
+int fused_variant(const Geom& g, int dir);
+FusedShape fused_shape(int dir, int variant);
+void launch_ac_fused(int dir, int variant, const AcFusedArgs& a, cudaStream_t st);
+
 // Setup (setup.cu)
 struct SetupArgs {
   Geom g;
