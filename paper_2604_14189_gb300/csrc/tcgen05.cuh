@@ -17,7 +17,9 @@
 //             MMA consumes 16 K lines: the k-th slice starts 16 k lines in.
 // The swizzle is a function of the shared-memory address, the same one TMA
 // applies when it writes a box with the matching swizzle mode, so every
-// operand buffer starts on a 1024-byte boundary.
+// operand buffer starts on a 1024-byte boundary; an operand may start on any
+// line of it (a shifted tap), and runs that LBO sets a line or a row apart
+// may overlap.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -30,7 +32,7 @@ namespace sweep {
 // Shared-memory matrix descriptor (tcgen05 format): start address, leading
 // and stride byte offsets (all >> 4), the fixed version field (1), base
 // offset 0 (atoms aligned), swizzle mode in bits 61..63.
-enum SmemSwizzle : uint32_t { kSwizzleNone = 0, kSwizzle128 = 2, kSwizzle64 = 4, kSwizzle32 = 6 };
+enum SmemSwizzle : uint32_t { kSwizzle128 = 2, kSwizzle64 = 4, kSwizzle32 = 6 };
 
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo,
                                               uint32_t swz) {
@@ -77,23 +79,40 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A * B^T, issued by one thread.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
+// One lane of a converged warp (the same one every time).
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(e));
+  return e;
 }
 
-// Arrive once on `bar` when every tcgen05 operation this thread issued so
-// far has completed.
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
+// D[tmem] (+)= A * B for one 16-deep K step, M and N as in idesc; called by a
+// converged warp and issued by the lane whose `e` is set (calls from inside a
+// branch on the lane index were issued more slowly).
+__device__ __forceinline__ void mma_bf16_warp(uint32_t e, uint32_t d_tmem, uint64_t adesc,
+                                              uint64_t bdesc, uint32_t idesc,
+                                              uint32_t accumulate) {
   asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(bar))
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(e)
+      : "memory");
+}
+// Arrive once on `bar` when every tcgen05 operation lane `e` issued so far has
+// completed.
+__device__ __forceinline__ void mma_commit_warp(uint32_t e, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
+          smem_u32(bar)),
+      "r"(e)
       : "memory");
 }
 

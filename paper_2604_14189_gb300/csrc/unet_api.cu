@@ -25,6 +25,9 @@ constexpr LayerDef kLayer[kUnetLayers] = {
     {128, 256}, {256, 256}, {256, 128}, {256, 128}, {128, 128}, {128, 64},
     {128, 64},  {64, 64},   {64, 32},   {64, 32},   {32, 32}};
 
+// level of each layer (H >> level, W >> level)
+constexpr int kLevel[kUnetLayers] = {0, 0, 1, 1, 2, 2, 3, 3, 2, 2, 2, 1, 1, 1, 0, 0, 0};
+
 long long layer_off(int l) {  // start of layer l's weights in the flat vector
   long long o = 0;
   for (int k = 0; k < l; ++k) o += (long long)kLayer[k].cout * 9 * kLayer[k].cin + kLayer[k].cout;
@@ -48,9 +51,7 @@ struct Bump {
   }
 };
 
-constexpr int kRedBlocks = 256;       // partial sums of the loss / head / bias reductions
-constexpr int kMaxWgradCtas = 512;    // split-K CTAs of one weight-gradient launch
-constexpr int kStages = 4;
+constexpr int kRedBlocks = 256;  // partial sums of the loss / head reductions
 
 bool pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
@@ -91,7 +92,15 @@ UnetLayout layout(const sweep_unet_shape* s, bool training) {
   L.status = b.take(sizeof(int) * 4);
   L.lpart = b.take(sizeof(double) * kRedBlocks + sizeof(float) * 33 * kRedBlocks);
   L.bpart = b.take(sizeof(float) * kRedBlocks * 256);
-  L.wpart = training ? b.take(sizeof(float) * (size_t)kMaxWgradCtas * 128 * 256) : 0;
+  size_t wpart = 0;  // the largest layer's partial sums
+  if (training)
+    for (int l = 0; l < kUnetLayers; ++l) {
+      size_t n = 0;
+      wgrad_plan(s->batch, s->height >> kLevel[l], s->width >> kLevel[l], kLayer[l].cin,
+                 kLayer[l].cout, &n);
+      wpart = std::max(wpart, n);
+    }
+  L.wpart = b.take(sizeof(float) * wpart);
   for (int l = 0; l < kUnetLayers; ++l) {
     const size_t n = (size_t)kLayer[l].cout * 9 * kLayer[l].cin * sizeof(bf16);
     L.w[l] = b.take(n);
@@ -128,15 +137,7 @@ struct View {
   int ps, C;
 };
 
-int kchunk(int c) { return c >= 64 ? 64 : 32; }
-
-// Pipeline depth of a convolution: as many stages (2..4) as let two CTAs
-// share an SM, so that one CTA's epilogue overlaps the other's main loop.
-int conv_stages(int cout, int kc) {
-  const int stage = 128 * kc * 2 + cout * kc * 2;
-  const int budget = 112 * 1024 - 1024;  // half an SM's shared memory
-  return std::max(2, std::min(kStages, budget / stage));
-}
+int kchunk(int c) { return c % 64 == 0 ? 64 : 32; }
 
 bool act_map(CUtensorMap* m, const View& v, int B, int H, int W, int kc, int bw, int bh) {
   const uint64_t dims[4] = {(uint64_t)v.C, (uint64_t)W, (uint64_t)H, (uint64_t)B};
@@ -145,11 +146,13 @@ bool act_map(CUtensorMap* m, const View& v, int B, int H, int W, int kc, int bw,
   return make_tensor_map_bf16(m, v.p, 4, dims, str, box, kc * 2);
 }
 
-bool weight_map(CUtensorMap* m, const bf16* w, int cin, int cout, int kc) {
-  const uint64_t dims[3] = {(uint64_t)cin, 9, (uint64_t)cout};
-  const uint64_t str[2] = {(uint64_t)cin, (uint64_t)cin * 9};
-  const uint32_t box[3] = {(uint32_t)kc, 1, (uint32_t)cout};
-  return make_tensor_map_bf16(m, w, 3, dims, str, box, kc * 2);
+// The maps of a convolution whose tile the launcher has chosen.
+bool conv_maps(ConvArgs& a) {
+  const uint64_t wd[3] = {(uint64_t)a.cin, 9, (uint64_t)a.cout};
+  const uint64_t ws[2] = {(uint64_t)a.cin, (uint64_t)a.cin * 9};
+  const uint32_t wb[3] = {(uint32_t)a.kc, 1, (uint32_t)a.n};
+  return act_map(&a.tin, {a.in, a.in_ps, a.cin}, a.B, a.H, a.W, a.kc, 8 * a.ns + 2, 18) &&
+         make_tensor_map_bf16(&a.tw, a.w, 3, wd, ws, wb, a.kc * 2);
 }
 
 // One convolution on an H x W level: in (cin channels) * w [cout][9][cin].
@@ -163,9 +166,6 @@ int run_conv(int B, int H, int W, const View& in, const bf16* w, int cin, int co
   a.cin = cin;
   a.cout = cout;
   a.kc = kchunk(cin);
-  a.bw = std::min(W, 128);
-  a.bh = 128 / a.bw;
-  a.stages = conv_stages(cout, a.kc);
   a.bias = bias;
   a.op = op;
   a.mask = mask;
@@ -173,44 +173,32 @@ int run_conv(int B, int H, int W, const View& in, const bf16* w, int cin, int co
   a.out = out;
   a.out_ps = out_ps;
   a.status = status;
-  if (H % a.bh != 0) return SWEEP_EINVAL;
-  if (!act_map(&a.tin, in, B, H, W, a.kc, a.bw, a.bh)) return SWEEP_ECUDA;
-  if (!weight_map(&a.tw, w, cin, cout, a.kc)) return SWEEP_ECUDA;
-  launch_conv(a, st);
-  return SWEEP_OK;
+  a.in = in.p;
+  a.in_ps = in.ps;
+  a.w = w;
+  a.make_maps = conv_maps;
+  return launch_conv(a, st);
 }
 
-int wgrad_splits(int mtiles, long long T) {
-  const int ctas = std::min(2 * device_sms(), kMaxWgradCtas);
-  long long s = std::max(1, ctas / mtiles);
-  s = std::min<long long>(s, T);
-  return (int)std::max<long long>(s, 1);
-}
-
-// dW (FP32 [cout][9][cin]) of one convolution; partial: the split sums.
+// dW (FP32 [cout][9][cin]) and, unless NULL, db of one convolution; partial,
+// bpart: the split sums.
 int run_wgrad(int B, int H, int W, const View& x, const View& dy, int cin, int cout, float* dW,
-              float* partial, int* status, cudaStream_t st) {
+              float* partial, float* bpart, float* db, int* status, cudaStream_t st) {
   WgradArgs a{};
+  a.plan = wgrad_plan(B, H, W, cin, cout, nullptr);
   a.B = B;
   a.H = H;
   a.W = W;
   a.cin = cin;
   a.cout = cout;
-  a.ka = kchunk(cin);
-  a.kb = kchunk(cout);
-  a.pw = std::min(W, 64);
-  a.ph = 64 / a.pw;
-  if (H % a.ph != 0) return SWEEP_EINVAL;
-  a.mtiles = (9 * cin + 127) / 128;
-  const long long T = (long long)B * (H / a.ph) * (W / a.pw);
-  a.splits = wgrad_splits(a.mtiles, T);
-  a.stages = kStages;
   a.partial = partial;
   a.status = status;
-  if (!act_map(&a.tin, x, B, H, W, a.ka, a.pw, a.ph)) return SWEEP_ECUDA;
-  if (!act_map(&a.tdy, dy, B, H, W, a.kb, a.pw, a.ph)) return SWEEP_ECUDA;
+  const int px = a.plan.q * a.plan.pw;  // of a stage's rows
+  if (!act_map(&a.tin, x, B, H, W, a.plan.kc, px + 2, a.plan.ph)) return SWEEP_ECUDA;
+  if (!act_map(&a.tdy, dy, B, H, W, a.plan.kb, px, a.plan.ph)) return SWEEP_ECUDA;
   launch_wgrad(a, st);
-  launch_wgrad_reduce(partial, a.splits, a.mtiles * 128, cin, cout, dW, st);
+  if (db) launch_bias_grad(dy.p, dy.ps, cout, (long long)B * H * W, bpart, kRedBlocks, st);
+  launch_wgrad_reduce(a, dW, bpart, kRedBlocks, db, st);
   return SWEEP_OK;
 }
 
@@ -241,12 +229,8 @@ struct Net {
   int wgrad(int level, const View& x, const View& dpre, int l, float* grad) {
     float* dW = grad + layer_off(l);
     const int cin = kLayer[l].cin, cout = kLayer[l].cout;
-    int rc = run_wgrad(B, h(level), w(level), x, dpre, cin, cout, dW, at<float>(ws, L.wpart),
-                       status, st);
-    if (rc) return rc;
-    launch_bias_grad(dpre.p, dpre.ps, cout, npix(level), at<float>(ws, L.bpart), kRedBlocks,
-                     dW + (long long)cout * 9 * cin, st);
-    return SWEEP_OK;
+    return run_wgrad(B, h(level), w(level), x, dpre, cin, cout, dW, at<float>(ws, L.wpart),
+                     at<float>(ws, L.bpart), dW + (long long)cout * 9 * cin, status, st);
   }
 };
 
@@ -446,7 +430,9 @@ extern "C" int sweep_unet_conv3x3(int32_t B, int32_t H, int32_t W, int32_t cin, 
 extern "C" size_t sweep_unet_wgrad_workspace_bytes(int32_t B, int32_t H, int32_t W,
                                                    int32_t cin, int32_t cout) {
   if (!single_conv_shape_ok(B, H, W, cin, cout, 64)) return 0;
-  return kAlign + sizeof(float) * (size_t)kMaxWgradCtas * 128 * 256;
+  size_t n = 0;
+  wgrad_plan(B, H, W, cin, cout, &n);
+  return kAlign + sizeof(float) * n;
 }
 
 extern "C" int sweep_unet_conv3x3_wgrad(int32_t B, int32_t H, int32_t W, int32_t cin,
@@ -462,6 +448,6 @@ extern "C" int sweep_unet_conv3x3_wgrad(int32_t B, int32_t H, int32_t W, int32_t
   float* partial = reinterpret_cast<float*>(static_cast<char*>(ws) + kAlign);
   UNET_TRY(run_wgrad(B, H, W, {reinterpret_cast<const bf16*>(x), cin, cin},
                      {reinterpret_cast<const bf16*>(dy), cout, cout}, cin, cout, dw, partial,
-                     status, st));
+                     nullptr, nullptr, status, st));
   return cudaGetLastError() == cudaSuccess ? SWEEP_OK : SWEEP_ECUDA;
 }

@@ -1,21 +1,32 @@
 // 3 x 3 convolutions of the U-Net preconditioner on the 5th-generation
 // tensor cores (tcgen05, BF16 operands, FP32 accumulator in tensor memory).
 //
-// conv_kernel: one CTA per 128-pixel output tile computes all output
-// channels: an implicit GEMM with M = 128 pixels, N = cout (<= 256), and
-// K = 9 taps x cin, walked in (tap, channel chunk) steps.  Warp 0 stages the
-// shifted input tile (a TMA box of the NHWC tensor at the tap's offset; the
-// zero padding is the box's out-of-bounds fill) and the weights' (tap,
-// chunk) slice into a 4-stage ring; warp 1 issues the MMAs of a stage
-// (one per 16 channels) and releases it with a commit; then all four warps
-// read the accumulator out of TMEM (one pixel per thread), add the bias,
-// apply ReLU or the ReLU mask of the backward pass, and store BF16.
+// conv_kernel: an implicit GEMM with M = 128 pixels per accumulator, N output
+// channels, and K = 9 taps x cin in (tap, channel chunk) order.  A CTA takes a
+// tile of 16 rows x 8, 16 or 32 columns (1, 2 or 4 accumulators) and all or
+// part of the output channels.  The input tile is staged once, with a
+// one-pixel halo (TMA boxes of the NHWC tensor; the zero padding is the box's
+// out-of-bounds fill), and a tap is an offset into it; the weights' (tap,
+// chunk) slices go through a ring.  What bounds it: MMAs into one accumulator
+// follow one another at about 146 cycles and an MMA of N <= 64 takes 44
+// cycles, whatever its N; a CTA's set-up, first loads and epilogue take about
+// 3 us.  So the launcher's cost model looks for several accumulators in
+// flight on an SM (of one CTA, or of several) before large tiles.  Staging a
+// shifted tile per tap with one accumulator per CTA read the input nine times
+// through L2: 8 x 256 x 256 pixels, 32 -> 32 channels, 40 us, now 23 (10 us
+// are the bytes at the copy rate); 8 x 64 x 64, 256 -> 128: 76 us, now 22;
+// 8 x 32 x 32, 256 -> 256: 25 us, now 15 (11 us are the chain of MMAs).
 //
-// wgrad_kernel: D[(tap, ci)][co] = sum over pixels of in[p + off(tap)][ci]
-// dy[p][co]; a CTA owns 128 rows of (tap, ci) and a contiguous range of
-// 64-pixel steps (split K); both operands are staged pixel-major by TMA,
-// i.e. MN-major for the MMA.  Each CTA writes its FP32 partial sums; a
-// reduction kernel adds the splits in a fixed order.
+// wgrad_kernel: the weight gradient, a split-K GEMM over the pixels (see
+// WgradPlan in unet_internal.cuh).  Both operands are staged pixel-major by TMA,
+// i.e. MN-major for the MMA; the input with a pixel more on either side, so that
+// the taps of a row are offsets into one staged box, and 128 pixels a stage
+// where the rows are that long.  Each CTA writes its FP32 partial sums; a
+// reduction kernel adds the splits in a fixed order.  Bound by the chain of
+// dependent MMAs of a split (146 cycles each: without any loads 8 x 256 x 256,
+// 32 -> 32 channels takes 31 us) and, close behind, by the lines that TMA
+// fetches.  Four boxes per 64 pixels and 128 (tap, ci) rows took 104 us there,
+// now 33; 64 -> 32 channels 142, now 56; 8 x 128 x 128, 128 -> 64: 69, now 33.
 //
 // Every mbarrier wait is bounded (tma.cuh); a wait that gives up latches
 // SWEEP_ETIMEOUT, the CTA skips its stores, waits for its own copies in
@@ -30,13 +41,13 @@
 namespace sweep {
 namespace {
 
-constexpr int kThreads = 128;
-constexpr int kMaxStages = 4;
+constexpr int kConvMaxStages = 24;
 constexpr size_t kSmemPerSm = 228 * 1024;  // per SM, of which 1 KB per CTA is reserved
-// dynamic shared memory the kernels may ask for: 4 stages of at most 48 KB
-// and the 1 KB alignment slack (below the 227 KB opt-in limit, which also
-// counts the kernels' static barriers)
-constexpr int kMaxDynSmem = 4 * 48 * 1024 + 1024;
+// dynamic shared memory a kernel may ask for (below the 227 KB opt-in limit,
+// which also counts the static barriers)
+constexpr int kConvMaxSmem = 225 * 1024;
+constexpr int kWgMaxSmem = 225 * 1024;
+constexpr int kWgMaxCtas = 512;
 
 __host__ __device__ inline uint32_t tmem_cols(int n) {
   uint32_t c = 32;
@@ -55,37 +66,75 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-__global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant__ ConvArgs a) {
-  __shared__ __align__(8) uint64_t full[kMaxStages];
-  __shared__ __align__(8) uint64_t empty[kMaxStages];
+// The values of w whose mask is positive, 0 for the others (8 BF16 each).
+__device__ __forceinline__ uint4 mask8(uint4 w, const uint4& m) {
+  __nv_bfloat16* v = reinterpret_cast<__nv_bfloat16*>(&w);
+  const __nv_bfloat16* k = reinterpret_cast<const __nv_bfloat16*>(&m);
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (!(__bfloat162float(k[i]) > 0.f)) v[i] = __float2bfloat16_rn(0.f);
+  return w;
+}
+
+// Convolution tile: 16 rows x 8 ns columns of pixels.  An accumulator takes
+// 128 of them (16 rows x 8 columns): the 8 pixels of a row are one 8-row core
+// matrix of the A operand, and SBO is the row pitch of the staged tile.
+constexpr int kConvRows = 16;
+constexpr int kConvThreads = 192;  // warps 0-3: epilogue, 4: TMA, 5: MMA
+constexpr int kMaxChunks = 8;      // input channel chunks
+
+// Bytes of a staged chunk of kc channels: a line of 2 kc bytes per pixel,
+// padded to whole swizzle atoms.
+__host__ __device__ inline uint32_t chunk_bytes(int ns, int kc) {
+  return (uint32_t)((8 * ns + 2) * (kConvRows + 2) * 2 * kc + 1023) / 1024 * 1024;
+}
+
+template <int KC, int NS>
+__global__ void __launch_bounds__(kConvThreads)
+    conv_kernel(const __grid_constant__ ConvArgs a) {
+  __shared__ __align__(8) uint64_t full[kConvMaxStages];
+  __shared__ __align__(8) uint64_t empty[kConvMaxStages];
+  __shared__ __align__(8) uint64_t inbar[kMaxChunks];
   __shared__ __align__(8) uint64_t done;
   __shared__ uint32_t tmem_holder;
   __shared__ int failed;
+  __shared__ __align__(16) float bias[256];
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_u = smem_u32(smem_raw);
   const uint32_t base_u = (raw_u + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (base_u - raw_u);
-  const int a_bytes = 128 * a.kc * 2;
-  const int stage_bytes = a_bytes + a.cout * a.kc * 2;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t ncols = tmem_cols(a.cout);
   const int S = a.stages;
+  const int PW = 8 * NS + 2;                              // staged pixels per row
+  const uint32_t CS = chunk_bytes(NS, KC);
+  const int nch = a.cin / KC, kiters = 9 * nch;
+  // the staged input, then the ring: weights and, when the input does not
+  // stay, a chunk of it behind them
+  const uint32_t wbytes = (uint32_t)(a.n * KC * 2), stage_bytes = wbytes + (a.stays ? 0 : CS);
+  const int kept = a.stays ? nch : 0;
+  const uint32_t in_u = base_u, ring_u = base_u + (uint32_t)kept * CS;
+  uint8_t* in = base;
+  base += (size_t)kept * CS;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const uint32_t ncols = tmem_cols(a.n * NS);
 
-  const int ntx = a.W / a.bw, nty = a.H / a.bh;
-  int t = blockIdx.x;
+  const int nblk = a.cout / a.n;
+  int t = blockIdx.x / nblk;
+  const int n0 = (blockIdx.x - t * nblk) * a.n;
+  const int ntx = a.W / (8 * NS), nty = (a.H + kConvRows - 1) / kConvRows;
   const int b = t / (ntx * nty);
   t -= b * ntx * nty;
-  const int y0 = (t / ntx) * a.bh, x0 = (t % ntx) * a.bw;
+  const int y0 = (t / ntx) * kConvRows, x0 = (t % ntx) * 8 * NS;
 
-  if (warp == 0) {
+  if (warp == 5) {
     tmem_alloc(&tmem_holder, ncols);
     tmem_relinquish();
   }
-  if (threadIdx.x == 32) {
+  if (threadIdx.x == 128) {
     for (int i = 0; i < S; ++i) {
       mbar_init(&full[i], 1);
       mbar_init(&empty[i], 1);
     }
+    for (int i = 0; i < kept; ++i) mbar_init(&inbar[i], 1);
     mbar_init(&done, 1);
     failed = 0;
     fence_barrier_init();
@@ -95,134 +144,218 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
   tc_fence_after();
   const uint32_t tmem = tmem_holder;
 
-  const int nch = a.cin / a.kc;
-  const int kiters = 9 * nch;
-  if (warp == 0) {  // TMA producer
-    int k = 0;
-    for (; k < kiters; ++k) {
-      const int s = k % S;
-      if (k >= S && !warp_wait(&empty[s], ((k / S) - 1) & 1)) {
-        if (lane == 0) {
+  if (warp == 4) {  // TMA producer
+    if (lane == 0) {
+      int k = 0, s = 0, ph = 1, tap = 0, ch = 0;  // (the ring's first pass waits for nothing)
+      for (; k < kiters; ++k) {
+        if (k < kept) {  // the input tile, chunk by chunk (zero off the image)
+          mbar_arrive_expect_tx(&inbar[k], (uint32_t)(PW * (kConvRows + 2) * 2 * KC));
+          tma_load_4d(in + (size_t)k * CS, &a.tin, &inbar[k], k * KC, x0 - 1, y0 - 1, b);
+        }
+        if (k >= S && !mbar_wait(&empty[s], ph)) {
           latch(a.status, SWEEP_ETIMEOUT);
           failed = 1;
+          break;
         }
-        break;
-      }
-      if (lane == 0) {
-        const int tap = k / nch, ch = k - tap * nch;
-        uint8_t* sa = base + (size_t)s * stage_bytes;
-        mbar_arrive_expect_tx(&full[s], stage_bytes);
-        tma_load_4d(sa, &a.tin, &full[s], ch * a.kc, x0 + tap % 3 - 1, y0 + tap / 3 - 1, b);
-        tma_load_3d(sa + a_bytes, &a.tw, &full[s], ch * a.kc, tap, 0);
-      }
-      __syncwarp();
-    }
-    // the last copy into each stage has landed before the CTA may exit
-    for (int j = k > S ? k - S : 0; j < k; ++j) warp_wait(&full[j % S], (j / S) & 1);
-  } else if (warp == 1) {  // MMA issuer
-    const uint32_t idesc = idesc_bf16_f32(128, a.cout, 0, 0);
-    const uint32_t swz = a.kc == 64 ? kSwizzle128 : kSwizzle64;
-    const uint32_t sbo = 8u * a.kc * 2u;
-    for (int k = 0; k < kiters; ++k) {
-      const int s = k % S;
-      if (!warp_wait(&full[s], (k / S) & 1)) {
-        if (lane == 0) {
-          latch(a.status, SWEEP_ETIMEOUT);
-          failed = 1;
+        uint8_t* st = base + (size_t)s * stage_bytes;
+        mbar_arrive_expect_tx(&full[s],
+                              wbytes + (a.stays ? 0 : (uint32_t)(PW * (kConvRows + 2) * 2 * KC)));
+        tma_load_3d(st, &a.tw, &full[s], ch * KC, tap, n0);
+        if (!a.stays) tma_load_4d(st + wbytes, &a.tin, &full[s], ch * KC, x0 - 1, y0 - 1, b);
+        if (++s == S) {
+          s = 0;
+          ph ^= 1;
         }
-        break;
+        if (++ch == nch) {
+          ch = 0;
+          ++tap;
+        }
       }
-      tc_fence_after();
-      if (lane == 0) {
-        const uint32_t sa = base_u + (uint32_t)(s * stage_bytes);
-        const uint32_t sb = sa + (uint32_t)a_bytes;
-        for (int j = 0; j < a.kc / 16; ++j)
-          mma_bf16(tmem, smem_desc(sa + 32u * j, 16u, sbo, swz),
-                   smem_desc(sb + 32u * j, 16u, sbo, swz), idesc, (k | j) != 0);
-        mma_commit(&empty[s]);  // the stage is free once these MMAs have read it
-      }
-      __syncwarp();
+      // every copy has landed before the CTA may exit
+      for (int j = k > S ? k - S : 0; j < k; ++j) mbar_wait(&full[j % S], (j / S) & 1);
+      for (int j = 0; j < min(k, kept); ++j) mbar_wait(&inbar[j], 0);
     }
-    if (lane == 0) mma_commit(&done);  // every MMA issued has completed
+    __syncwarp();
+  } else if (warp == 5) {  // MMA issuer (the whole warp, one lane issuing)
+    const uint32_t e = elect_one();
+    const uint32_t idesc = idesc_bf16_f32(128, a.n, 0, 0);
+    const uint32_t swz = KC == 64 ? kSwizzle128 : kSwizzle64;
+    const uint32_t line = 2u * KC;  // bytes of a staged pixel
+    const uint64_t adesc = smem_desc(in_u, 16u, (uint32_t)PW * line, swz);
+    const uint64_t bdesc = smem_desc(ring_u, 16u, 8u * KC * 2u, swz);
+    int s = 0, ph = 0;
+    bool ok = true;
+    for (int tap = 0; tap < 9 && ok; ++tap) {
+      // (addresses are the descriptors' low bits, in 16 bytes)
+      const uint64_t shift = (uint64_t)((uint32_t)(tap / 3 * PW + tap % 3) * (line >> 4));
+      uint64_t at = adesc + shift;
+      for (int ch = 0; ch < nch; ++ch) {
+        ok = mbar_wait(&full[s], ph) && (tap > 0 || !a.stays || mbar_wait(&inbar[ch], 0));
+        if (!__all_sync(0xffffffffu, ok)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint64_t bd = bdesc + (uint64_t)((uint32_t)s * stage_bytes >> 4);
+        if (!a.stays) at = adesc + shift + (uint64_t)(((uint32_t)s * stage_bytes + wbytes) >> 4);
+#pragma unroll
+        for (int j = 0; j < KC / 16; ++j)
+#pragma unroll
+          for (int q = 0; q < NS; ++q)
+            mma_bf16_warp(e, tmem + (uint32_t)(q * a.n), at + 2 * j + (line >> 1) * q, bd + 2 * j,
+                          idesc, (tap | ch | j) != 0);
+        mma_commit_warp(e, &empty[s]);  // the stage is free once these MMAs have read it
+        at += CS >> 4;
+        if (++s == S) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+    }
+    if (!ok && lane == 0) {
+      latch(a.status, SWEEP_ETIMEOUT);
+      failed = 1;
+    }
+    mma_commit_warp(e, &done);  // every MMA issued has completed
     __syncwarp();
   }
 
+  // The epilogue.  A lane holds 32 channels of pixel (row 4 warp + lane / 8,
+  // column lane % 8) of its accumulator; through shared memory (the staged
+  // input's, free by then) four lanes take the 64 bytes of a pixel, so that a
+  // store covers whole sectors.  The bias and the first step's mask are read
+  // while the MMAs run, a step's mask while the step before it is stored.
+  const int px = lane >> 2, cu = lane & 3, steps = NS * (a.n / 32);
+  const long long pix0 = ((long long)b * a.H + y0 + 4 * warp) * a.W + x0 + px;
+  uint4 mk[4];
+  auto load_mask = [&](int q, int c0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (y0 + 4 * warp + i < a.H)
+        mk[i] = *reinterpret_cast<const uint4*>(
+            a.mask + (pix0 + 8 * q + (long long)i * a.W) * a.mask_ps + n0 + c0 + 8 * cu);
+  };
+  if (warp < 4) {
+    if (a.bias)
+      for (int i = threadIdx.x; i < a.n; i += 128) bias[i] = a.bias[n0 + i];
+    if (a.op == kOpMask) load_mask(0, 0);
+  }
   const bool got = mbar_wait(&done, 0);
   const bool bad = __syncthreads_or(!got) || failed;
   tc_fence_after();
-  if (!bad && kiters > 0) {
-    const int r = warp * 32 + lane;  // accumulator lane = output pixel of the tile
-    const long long pix = ((long long)b * a.H + (y0 + r / a.bw)) * a.W + (x0 + r % a.bw);
-    bf16* op = a.out + pix * a.out_ps;
-    const bf16* mp = a.op == kOpMask ? a.mask + pix * a.mask_ps : nullptr;
-    for (int c0 = 0; c0 < a.cout; c0 += 32) {
+  if (!bad && warp < 4) {
+    uint8_t* xch = in + warp * 2048;
+    int q = 0, c0 = 0;
+    for (int k = 0; k < steps; ++k) {
       float v[32];
-      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(q * a.n + c0), v);
       if (a.bias) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] += a.bias[c0 + i];
+        for (int i = 0; i < 8; ++i) {
+          const float4 f = *reinterpret_cast<const float4*>(bias + c0 + 4 * i);
+          v[4 * i] += f.x;
+          v[4 * i + 1] += f.y;
+          v[4 * i + 2] += f.z;
+          v[4 * i + 3] += f.w;
+        }
       }
       if (a.op == kOpRelu) {
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] = fmaxf(v[i], 0.f);
-      } else if (a.op == kOpMask) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint4 m = *reinterpret_cast<const uint4*>(mp + c0 + 8 * q);
-          const bf16* mb = reinterpret_cast<const bf16*>(&m);
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            if (!(__bfloat162float(mb[i]) > 0.f)) v[8 * q + i] = 0.f;
-        }
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int u = 0; u < 4; ++u) {
         uint4 w;
-        w.x = pack2(v[8 * q + 0], v[8 * q + 1]);
-        w.y = pack2(v[8 * q + 2], v[8 * q + 3]);
-        w.z = pack2(v[8 * q + 4], v[8 * q + 5]);
-        w.w = pack2(v[8 * q + 6], v[8 * q + 7]);
-        *reinterpret_cast<uint4*>(op + c0 + 8 * q) = w;
+        w.x = pack2(v[8 * u + 0], v[8 * u + 1]);
+        w.y = pack2(v[8 * u + 2], v[8 * u + 3]);
+        w.z = pack2(v[8 * u + 4], v[8 * u + 5]);
+        w.w = pack2(v[8 * u + 6], v[8 * u + 7]);
+        *reinterpret_cast<uint4*>(xch + lane * 64 + ((u ^ (lane >> 1)) & 3) * 16) = w;
       }
+      __syncwarp();
+      bf16* o = a.out + (pix0 + 8 * q) * a.out_ps + n0 + c0 + 8 * cu;
+      uint4 w[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int p = 8 * i + px;
+        w[i] = *reinterpret_cast<const uint4*>(xch + p * 64 + ((cu ^ (p >> 1)) & 3) * 16);
+        if (a.op == kOpMask) w[i] = mask8(w[i], mk[i]);
+      }
+      if ((c0 += 32) == a.n) {
+        c0 = 0;
+        ++q;
+      }
+      if (a.op == kOpMask && k + 1 < steps) load_mask(q, c0);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (y0 + 4 * warp + i < a.H)
+          *reinterpret_cast<uint4*>(o + (long long)i * a.W * a.out_ps) = w[i];
+      __syncwarp();
     }
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (warp == 5) {
     tc_fence_after();
     tmem_dealloc(tmem, ncols);
   }
 }
 
-__global__ void __launch_bounds__(kThreads, 1) wgrad_kernel(const __grid_constant__ WgradArgs a) {
-  __shared__ __align__(8) uint64_t full[kMaxStages];
-  __shared__ __align__(8) uint64_t empty[kMaxStages];
+constexpr int kWgMaxUnits = 3;  // of a CTA
+constexpr int kWgMaxStages = 16;
+
+// Bytes of a staged chunk of kc channels: ph rows of q pw + 2 pixels, in whole
+// swizzle atoms (a unit's unused runs read past it, into what lies behind).
+__host__ __device__ inline uint32_t wg_chunk_bytes(const WgradPlan& P) {
+  return (uint32_t)(P.ph * (P.q * P.pw + 2) * 2 * P.kc + 1023) / 1024 * 1024;
+}
+// Rows of strips that a set stages (ky from its first unit's to its last's).
+__host__ __device__ inline int wg_rows(const WgradPlan& P, const WgradSet& w) {
+  const int c = wgrad_chunks(P, w.block);
+  const WgradUnit l = wgrad_unit(P, c, w.u1 - 1);
+  int hi = l.ky + l.down;
+  for (int u = w.u0; u < w.u1; ++u) {
+    const WgradUnit n = wgrad_unit(P, c, u);
+    hi = n.ky + n.down > hi ? n.ky + n.down : hi;
+  }
+  return hi - wgrad_unit(P, c, w.u0).ky + 1;
+}
+
+__global__ void __launch_bounds__(kConvThreads, 2)
+    wgrad_kernel(const __grid_constant__ WgradArgs a) {
+  __shared__ __align__(8) uint64_t full[kWgMaxStages];
+  __shared__ __align__(8) uint64_t empty[kWgMaxStages];
   __shared__ __align__(8) uint64_t done;
   __shared__ uint32_t tmem_holder;
   __shared__ int failed;
   extern __shared__ uint8_t smem_raw[];
+  const WgradPlan& P = a.plan;
   const uint32_t raw_u = smem_u32(smem_raw);
   const uint32_t base_u = (raw_u + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (base_u - raw_u);
-  constexpr int kPix = 64;                // K per stage (pixels)
-  constexpr int a_bytes = 128 * kPix * 2;  // 128 rows of (tap, ci) x 64 pixels
-  const int stage_bytes = a_bytes + a.cout * kPix * 2;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t ncols = tmem_cols(a.cout);
-  const int S = a.stages;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const uint32_t ncols = tmem_cols(P.per * a.cout);
 
-  const int mt = blockIdx.x % a.mtiles, split = blockIdx.x / a.mtiles;
-  const int ntx = a.W / a.pw, nty = a.H / a.ph;
+  // this CTA's set (input channel block, units) and its strips
+  const int split = blockIdx.x / P.sets, set = blockIdx.x - split * P.sets;
+  const WgradSet w = wgrad_set(P, set);
+  const int chunks = wgrad_chunks(P, w.block), nu = w.u1 - w.u0, rows = wg_rows(P, w);
+  const int ky0 = wgrad_unit(P, chunks, w.u0).ky;
+  const uint32_t CS = wg_chunk_bytes(P), DS = (uint32_t)(P.q * kWgPix * 2 * P.kb);
+  const uint32_t in_bytes = (uint32_t)(rows * chunks) * CS;
+  const uint32_t dy_bytes = (uint32_t)(P.q * kWgPix * 2 * a.cout);
+  const uint32_t stage_bytes = in_bytes + dy_bytes;
+  const int S = min(kWgMaxStages, P.ring / (int)stage_bytes);
+  const int ntx = a.W / P.pw, nty = a.H / P.ph;
   const long long T = (long long)a.B * ntx * nty;
-  const long long t0 = T * split / a.splits, t1 = T * (split + 1) / a.splits;
-  const int kiters = (int)(t1 - t0);
-  const int rows = 9 * a.cin;
+  const long long t0 = T * split / P.splits;
+  const int strips = (int)(T * (split + 1) / P.splits - t0);
 
-  if (warp == 0) {
+  if (warp == 5) {
     tmem_alloc(&tmem_holder, ncols);
     tmem_relinquish();
   }
-  if (threadIdx.x == 32) {
+  if (threadIdx.x == 128) {
     for (int i = 0; i < S; ++i) {
       mbar_init(&full[i], 1);
       mbar_init(&empty[i], 1);
@@ -236,137 +369,251 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_kernel(const __grid_constan
   tc_fence_after();
   const uint32_t tmem = tmem_holder;
 
-  if (warp == 0) {  // TMA producer
-    int k = 0;
-    for (; k < kiters; ++k) {
-      const int s = k % S;
-      if (k >= S && !warp_wait(&empty[s], ((k / S) - 1) & 1)) {
-        if (lane == 0) {
+  if (warp == 4) {  // TMA producer
+    if (lane == 0) {
+      const uint32_t bytes =
+          (uint32_t)(rows * chunks * P.ph * (P.q * P.pw + 2) * 2 * P.kc) + dy_bytes;
+      int k = 0, s = 0, ph = 1;
+      int tx = (int)(t0 % ntx), ty = (int)(t0 / ntx % nty), b = (int)(t0 / ntx / nty);
+      for (int left = strips; left > 0; ++k) {
+        if (k >= S && !mbar_wait(&empty[s], ph)) {
           latch(a.status, SWEEP_ETIMEOUT);
           failed = 1;
+          break;
         }
-        break;
-      }
-      if (lane == 0) {
-        long long tt = t0 + k;
-        const int b = (int)(tt / (ntx * nty));
-        tt -= (long long)b * ntx * nty;
-        const int y0 = (int)(tt / ntx) * a.ph, x0 = (int)(tt % ntx) * a.pw;
-        uint8_t* sa = base + (size_t)s * stage_bytes;
-        mbar_arrive_expect_tx(&full[s], stage_bytes);
-        for (int q = 0; q < 128 / a.ka; ++q) {  // runs of ka rows: one (tap, ci chunk) each
-          const int r0 = mt * 128 + q * a.ka;
-          int tap = r0 / a.cin, ci0 = r0 - tap * a.cin;
-          if (tap > 8) {  // rows past 9 cin: any valid tap; their sums are not stored
-            tap = 8;
-            ci0 = 0;
+        uint8_t* st = base + (size_t)s * stage_bytes;
+        mbar_arrive_expect_tx(&full[s], bytes);
+        for (int r = 0; r < rows; ++r)
+          for (int c = 0; c < chunks; ++c)
+            tma_load_4d(st + (size_t)(r * chunks + c) * CS, &a.tin, &full[s],
+                        (w.block * P.cpb + c) * P.kc, P.pw * tx - 1, P.ph * ty + ky0 + r - 1, b);
+        for (int q = 0; q < a.cout / P.kb; ++q)
+          tma_load_4d(st + in_bytes + (size_t)q * DS, &a.tdy, &full[s], q * P.kb, P.pw * tx,
+                      P.ph * ty, b);
+        if (++s == S) {
+          s = 0;
+          ph ^= 1;
+        }
+        const int n = min(min(P.q, ntx - tx), left);  // strips of this stage, of one row
+        left -= n;
+        if ((tx += n) == ntx) {
+          tx = 0;
+          if (++ty == nty) {
+            ty = 0;
+            ++b;
           }
-          tma_load_4d(sa + q * (kPix * a.ka * 2), &a.tin, &full[s], ci0, x0 + tap % 3 - 1,
-                      y0 + tap / 3 - 1, b);
         }
-        for (int q = 0; q < a.cout / a.kb; ++q)
-          tma_load_4d(sa + a_bytes + q * (kPix * a.kb * 2), &a.tdy, &full[s], q * a.kb, x0, y0,
-                      b);
       }
-      __syncwarp();
+      for (int j = k > S ? k - S : 0; j < k; ++j) mbar_wait(&full[j % S], (j / S) & 1);
     }
-    for (int j = k > S ? k - S : 0; j < k; ++j) warp_wait(&full[j % S], (j / S) & 1);
-  } else if (warp == 1) {  // MMA issuer: both operands MN-major
+    __syncwarp();
+  } else if (warp == 5) {  // MMA issuer: both operands MN-major, 16 pixels of a row per MMA
+    const uint32_t e = elect_one();
     const uint32_t idesc = idesc_bf16_f32(128, a.cout, 1, 1);
-    const uint32_t swa = a.ka == 64 ? kSwizzle128 : kSwizzle64;
-    const uint32_t swb = a.kb == 64 ? kSwizzle128 : kSwizzle64;
-    const uint32_t la = kPix * a.ka * 2, sba = 8u * a.ka * 2u;  // run stride, 8-line stride
-    const uint32_t lb = kPix * a.kb * 2, sbb = 8u * a.kb * 2u;
-    for (int k = 0; k < kiters; ++k) {
-      const int s = k % S;
-      if (!warp_wait(&full[s], (k / S) & 1)) {
-        if (lane == 0) {
-          latch(a.status, SWEEP_ETIMEOUT);
-          failed = 1;
-        }
+    const uint32_t la = 2u * P.kc, lb = 2u * P.kb;  // bytes of a staged pixel
+    const uint64_t b0 = smem_desc(base_u + in_bytes, DS, 8u * lb,
+                                  P.kb == 64 ? kSwizzle128 : kSwizzle64);
+    uint64_t a0[kWgMaxUnits];
+#pragma unroll
+    for (int u = 0; u < kWgMaxUnits; ++u) {
+      const WgradUnit n = wgrad_unit(P, chunks, min(w.u0 + u, w.u1 - 1));
+      a0[u] = smem_desc(base_u + (uint32_t)((n.ky - ky0) * chunks) * CS + (uint32_t)n.kx * la,
+                        chunks > 1 || n.down ? CS : la, 8u * la,
+                        P.kc == 64 ? kSwizzle128 : kSwizzle64);
+    }
+    int s = 0, ph = 0, tx = (int)(t0 % ntx);
+    uint32_t acc = 0;
+    bool ok = true;
+    for (int left = strips; left > 0;) {
+      ok = mbar_wait(&full[s], ph);
+      if (!__all_sync(0xffffffffu, ok)) {
+        ok = false;
         break;
       }
       tc_fence_after();
-      if (lane == 0) {
-        const uint32_t sa = base_u + (uint32_t)(s * stage_bytes);
-        const uint32_t sb = sa + (uint32_t)a_bytes;
-        for (int j = 0; j < kPix / 16; ++j)  // 16 pixels (K lines) per MMA
-          mma_bf16(tmem, smem_desc(sa + 16u * j * a.ka * 2u, la, sba, swa),
-                   smem_desc(sb + 16u * j * a.kb * 2u, lb, sbb, swb), idesc, (k | j) != 0);
-        mma_commit(&empty[s]);
+      const uint64_t so = (uint64_t)((uint32_t)s * stage_bytes >> 4);
+      const int n = min(min(P.q, ntx - tx), left);
+      left -= n;
+      tx = tx + n == ntx ? 0 : tx + n;
+      for (int h = 0; h < n; ++h) {
+#pragma unroll
+        for (int j = 0; j < kWgPix / 16; ++j) {
+          // (a strip of several rows is a stage of its own: h = 0)
+          const uint32_t px = (uint32_t)(kWgPix * h + 16 * j + 2 * (16 * j / P.pw));
+          const uint64_t ao = so + (uint64_t)(px * la >> 4);
+          const uint64_t br = b0 + so + (uint64_t)((uint32_t)(kWgPix * h + 16 * j) * lb >> 4);
+#pragma unroll
+          for (int u = 0; u < kWgMaxUnits; ++u)
+            if (u < nu)
+              mma_bf16_warp(e, tmem + (uint32_t)(u * a.cout), a0[u] + ao, br, idesc, acc);
+          acc = 1;
+        }
       }
-      __syncwarp();
+      mma_commit_warp(e, &empty[s]);
+      if (++s == S) {
+        s = 0;
+        ph ^= 1;
+      }
     }
-    if (lane == 0) mma_commit(&done);
+    if (!ok && lane == 0) {
+      latch(a.status, SWEEP_ETIMEOUT);
+      failed = 1;
+    }
+    mma_commit_warp(e, &done);
     __syncwarp();
   }
 
   const bool got = mbar_wait(&done, 0);
   const bool bad = __syncthreads_or(!got) || failed;
   tc_fence_after();
-  if (!bad) {
-    const int r = warp * 32 + lane;
-    const int R = mt * 128 + r;
-    float* out = a.partial + ((size_t)split * a.mtiles * 128 + R) * a.cout;
-    for (int c0 = 0; c0 < a.cout; c0 += 32) {
-      float v[32];
-      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);  // all lanes
-      if (R < rows) {
+  if (!bad && warp < 4) {
+    // a warp stores 32 rows of a column
+    float* out = a.partial + (size_t)blockIdx.x * P.per * a.cout * 128 + warp * 32 + lane;
+    for (int u = 0; u < nu; ++u)
+      for (int c0 = 0; c0 < a.cout; c0 += 32) {
+        float v[32];
+        tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(u * a.cout + c0), v);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          float4 w = kiters > 0 ? make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3])
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-          *reinterpret_cast<float4*>(out + c0 + 4 * q) = w;
-        }
+        for (int i = 0; i < 32; ++i) out[((size_t)u * a.cout + c0 + i) * 128] = v[i];
       }
-    }
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (warp == 5) {
     tc_fence_after();
     tmem_dealloc(tmem, ncols);
   }
 }
 
-// Shared memory of a launch, raised if needed so that the CTAs that fit on
-// one SM by shared memory never ask for more than the 512 TMEM columns.
-size_t fit_tmem(size_t smem, int cout) {
-  const size_t max_ctas = 512 / tmem_cols(cout);
-  // with at least this much each, max_ctas + 1 CTAs do not fit on one SM
-  const size_t floor_bytes = kSmemPerSm / (max_ctas + 1) + 1;
-  return std::max(smem, floor_bytes);
-}
-
 }  // namespace
 
-size_t conv_smem_bytes(int cout, int kc, int stages) {
-  const size_t s = (size_t)stages * (128 * kc * 2 + (size_t)cout * kc * 2) + 1024;
-  return fit_tmem(s, cout);
+// A convolution launch with tile width 8 ns and n output channels per CTA:
+// its weight stages, shared memory and estimated cycles (0: does not fit).
+// As many CTAs per SM as leave each a few stages (they hide one another's
+// set-up and epilogue), then as many stages as fit (small ones need many: a
+// stage takes a microsecond to arrive).  The estimate of a wave: its K steps
+// at the larger of the latency of dependent MMAs and the SM's tensor work,
+// plus set-up and epilogue.  Against a sweep of every (ns, n, CTAs per SM) on
+// 32 layers from 1 x 16 x 16 to 8 x 256 x 256 it picks the fastest or one
+// within 12 %; a fixed ns = 1, n = cout takes 1.3 to 2.2 times as long from
+// 8 x 64 x 64 up, a fixed ns = 4 1.2 to 1.6 times below.  stays: false stages
+// the input again for every tap, for inputs whose tile does not fit.
+struct ConvFit {
+  int ns, n;
+  bool stays;
+  int stages, ctas;
+  size_t smem;
+  double cycles;
+};
+constexpr double kConvChain = 146;   // cycles between MMAs into one accumulator
+constexpr double kConvFixed = 6000;  // set-up, first loads, drain
+constexpr double kConvOut = 16;      // epilogue, per output channel of an accumulator
+ConvFit conv_fit(const ConvArgs& a, int ns, int n, bool stays) {
+  ConvFit f{ns, n, stays, 0, 0, 0, 0.0};
+  const int chunks = a.cin / a.kc, kiters = 9 * chunks;
+  const size_t chunk = chunk_bytes(ns, a.kc), in = 1024 + (stays ? chunk * chunks : 0);
+  const size_t stage = (size_t)n * a.kc * 2 + (stays ? 0 : chunk);
+  const int cols = (int)tmem_cols(n * ns);
+  if (cols > 512 || (stays && chunks > kMaxChunks)) return f;
+  f.ctas = a.B * ((a.H + kConvRows - 1) / kConvRows) * (a.W / (8 * ns)) * (a.cout / n);
+  const int sms = device_sms(), per_sm = (f.ctas + sms - 1) / sms;
+  for (int res = std::max(1, std::min({512 / cols, per_sm, 4})); res >= 1; --res) {
+    const size_t budget = std::min<size_t>(kSmemPerSm / res - 3072, kConvMaxSmem);
+    if (budget < in + 2 * stage) continue;
+    const int s = (int)std::min<size_t>(kConvMaxStages, (budget - in) / stage);
+    if (res > 1 && s < std::min(3, kiters)) continue;
+    f.stages = std::min(s, kiters);
+    // no more CTAs on an SM than have tensor memory
+    f.smem = std::max(in + f.stages * stage, kSmemPerSm / (512 / cols + 1) + 1);
+    const double k = kiters * (a.kc / 16);
+    const double mma = std::max(40.0, 0.6 * n);
+    const int waves = (per_sm + res - 1) / res, last = per_sm - (waves - 1) * res;
+    const double step = std::max(kConvChain, ns * res * mma);
+    f.cycles = (waves - 1) * (k * step + kConvFixed) +
+               k * std::max(kConvChain, ns * last * mma) + kConvFixed + ns * n * kConvOut * waves;
+    return f;
+  }
+  return f;
 }
 
-size_t wgrad_smem_bytes(int cout, int stages) {
-  const size_t s = (size_t)stages * (128 * 64 * 2 + (size_t)cout * 64 * 2) + 1024;
-  return fit_tmem(s, cout);
-}
+void (*const kConvKernels[])(const ConvArgs) = {conv_kernel<32, 1>, conv_kernel<32, 2>,
+                                                conv_kernel<32, 4>, conv_kernel<64, 1>,
+                                                conv_kernel<64, 2>, conv_kernel<64, 4>};
 
-void launch_conv(const ConvArgs& a, cudaStream_t st) {
+int launch_conv(ConvArgs a, cudaStream_t st) {
   static std::once_flag once;
   std::call_once(once, [] {
-    cudaFuncSetAttribute(conv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+    for (auto* f : kConvKernels)
+      cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvMaxSmem);
   });
-  const int tiles = a.B * (a.H / a.bh) * (a.W / a.bw);
-  if (tiles <= 0) return;
-  conv_kernel<<<tiles, kThreads, conv_smem_bytes(a.cout, a.kc, a.stages), st>>>(a);
+  ConvFit best{};
+  for (const bool stays : {true, false}) {  // (false when nothing else fits)
+    for (int ns = 1; ns <= 4 && 8 * ns <= a.W; ns *= 2)
+      for (int n = 32; n <= std::min(a.cout, 256); n += 32) {
+        if (a.cout % n) continue;
+        const ConvFit f = conv_fit(a, ns, n, stays);
+        if (f.cycles > 0 && (best.cycles == 0 || f.cycles < best.cycles)) best = f;
+      }
+    if (best.cycles > 0) break;
+  }
+  if (best.cycles == 0) return SWEEP_EUNSUPPORTED;
+  a.ns = best.ns;
+  a.n = best.n;
+  a.stays = best.stays;
+  a.stages = best.stages;
+  if (!a.make_maps(a)) return SWEEP_ECUDA;
+  auto* kernel = kConvKernels[(a.kc == 64 ? 3 : 0) + (a.ns == 4 ? 2 : a.ns - 1)];
+  kernel<<<best.ctas, kConvThreads, best.smem, st>>>(a);
   note_launches(1);
+  return SWEEP_OK;
+}
+
+// The cut of a weight gradient.  Splits: as many as give 2 CTAs per SM with 128
+// rows of (tap, ci) each (at most kWgMaxCtas CTAs).  One unit per CTA: sets of
+// the units that share a staged row load less but leave SMs idle (8 x 256 x 256,
+// 32 -> 32: 43 us for 33; 64 -> 32: 103 for 56; others within 10 %).  partial:
+// floats of the partial sums.
+WgradPlan wgrad_plan(int B, int H, int W, int cin, int cout, size_t* partial) {
+  WgradPlan P{};
+  P.kc = cin % 64 == 0 ? 64 : 32;
+  P.kb = cout % 64 == 0 ? 64 : 32;
+  P.nchunks = cin / P.kc;
+  P.cpb = 128 / P.kc;
+  P.blocks = (P.nchunks + P.cpb - 1) / P.cpb;
+  P.pw = std::min(W, kWgPix);
+  P.ph = kWgPix / P.pw;
+  P.q = W >= 2 * kWgPix ? 2 : 1;  // (1 for all: 46 us for 33, 88 for 56, as above)
+  P.per = 1;
+  P.sets = (P.blocks - 1) * wgrad_block_sets(P, 0) + wgrad_block_sets(P, P.blocks - 1);
+  const long long T = (long long)B * (H / P.ph) * (W / P.pw);
+  const int mtiles = (9 * cin + 127) / 128;
+  P.splits = std::max(1, std::min(2 * device_sms(), kWgMaxCtas) / mtiles);
+  P.splits = (int)std::max(1LL, std::min<long long>(P.splits, T));
+  size_t staged = 0;  // most of a set's
+  for (int i = 0; i < P.sets; ++i) {
+    const WgradSet w = wgrad_set(P, i);
+    staged = std::max(staged, (size_t)wg_rows(P, w) * wgrad_chunks(P, w.block) * wg_chunk_bytes(P));
+  }
+  const size_t stage = staged + (size_t)P.q * kWgPix * 2 * cout;
+  // (the unused runs of a short block's units read past the last stage)
+  const int last = wgrad_chunks(P, P.blocks - 1);
+  const size_t slack = 1024 + (last > 1 ? (size_t)(P.cpb - last) * wg_chunk_bytes(P) : 0);
+  const int cols = (int)tmem_cols(P.per * cout);
+  const int res = cols <= 256 && slack + 2 * stage <= 110 * 1024 ? 2 : 1;
+  const size_t most = res == 2 ? 110 * 1024 : kWgMaxSmem;
+  P.ring = (int)std::min(most - slack, kWgMaxStages * stage);
+  P.smem = std::max(slack + P.ring, kSmemPerSm / (512 / cols + 1) + 1);
+  if (partial) *partial = (size_t)P.splits * P.sets * P.per * cout * 128;
+  return P;
 }
 
 void launch_wgrad(const WgradArgs& a, cudaStream_t st) {
   static std::once_flag once;
   std::call_once(once, [] {
-    cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+    cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgMaxSmem);
   });
-  wgrad_kernel<<<a.mtiles * a.splits, kThreads, wgrad_smem_bytes(a.cout, a.stages), st>>>(a);
+  const WgradPlan& P = a.plan;
+  wgrad_kernel<<<P.splits * P.sets, kConvThreads, P.smem, st>>>(a);
   note_launches(1);
 }
 

@@ -20,46 +20,114 @@ typedef __nv_bfloat16 bf16;
 
 // One 3 x 3 convolution as an implicit GEMM on the tensor cores:
 //   out[p][n] = op( sum_{tap, k} in[p + off(tap)][k] * w[n][tap][k] + bias[n] )
-// over 128-pixel tiles (M = 128 pixels, N = all output channels, K = 9
-// taps x input channels in chunks of kc).  The data gradient of a
+// over tiles of 16 x 8 ns pixels (M = 128 pixels each, N = n output channels,
+// K = 9 taps x input channels in chunks of kc).  The data gradient of a
 // convolution is the same operation on the output gradient with the
 // weights transposed and mirrored (w'[ci][8 - tap][co] = w[co][tap][ci]).
 enum ConvOp { kOpNone = 0, kOpRelu = 1, kOpMask = 2 };
 struct ConvArgs {
-  CUtensorMap tin;   // input view {cin, W, H, B}, box {kc, bw, bh, 1}
-  CUtensorMap tw;    // weights {cin, 9, cout}, box {kc, 1, cout}
+  CUtensorMap tin;   // input view {cin, W, H, B}, box {kc, 8 ns + 2, 18, 1}
+  CUtensorMap tw;    // weights {cin, 9, cout}, box {kc, 1, n}
   int B, H, W;
-  int cin, cout, kc;  // kc = 64 (128-byte swizzle) or 32 (64-byte)
-  int bw, bh;         // pixel tile: bw x bh = 128
-  int stages;
+  int cin, cout, kc;  // kc = 64 (128-byte swizzle of the weights) or 32 (64-byte)
+  int n, ns;          // a CTA's output channels and 8-pixel column groups
+  int stages;         // of the ring
+  int stays;          // the input tile is staged once (else once per tap)
   const float* bias;  // [cout] or NULL
   int op;             // ConvOp
+  const bf16* in;
+  int in_ps;
   const bf16* mask;   // kOpMask: out *= (mask > 0), same pixel/channel
   int mask_ps;
   bf16* out;
   int out_ps;
   int* status;        // latched on a wait that gives up
+  // what the launcher makes the maps from once it has chosen n and ns
+  const bf16* w;
+  bool (*make_maps)(ConvArgs&);
 };
 
 // Weight gradient of one 3 x 3 convolution on the tensor cores:
-//   D[(tap, ci)][co] = sum_p in[p + off(tap)][ci] * dy[p][co]
-// (M = 128 rows of (tap, ci) per CTA, N = cout, K = pixels in 64-pixel
-// steps, both operands MN-major), one partial sum per pixel split.
+//   D[(tap, ci)][co] = sum over pixels p of in[p + off(tap)][ci] dy[p][co]
+// (both operands MN-major, K = 16 pixels of a row per MMA).  The pixels are
+// taken in raster order, in strips of 64, and split into equal ranges; a range
+// is one accumulation, and the ranges' sums are added in a fixed order, so the
+// split is part of the result.  Within a split the work is cut by taps: a unit
+// is one accumulator of 128 rows made of 128 / kc runs of kc channels, of up to
+// cpb = 128 / kc channel chunks (a block):
+//   several chunks (9 units): unit = tap, run j = chunk j;
+//   one chunk of 64 (5 units): two taps: a pixel apart (kx = 0, 1) or a row
+//   apart (kx = 2);
+//   one chunk of 32 (3 units): unit = ky, runs a pixel apart (kx = 0, 1, 2).
+// A set is up to `per` units of a block; a CTA does one set of one split.
+constexpr int kWgPix = 64;  // pixels of a strip
+struct WgradPlan {
+  int kc, nchunks, cpb, blocks;  // input channels
+  int kb;                        // output channels per staged box
+  int pw, ph, q;                 // columns and rows of a strip, strips of a stage
+  int per, sets, splits;
+  int ring;      // bytes of a CTA's stages
+  size_t smem;
+};
+__host__ __device__ inline int wgrad_chunks(const WgradPlan& P, int block) {
+  const int n = P.nchunks - block * P.cpb;
+  return n < P.cpb ? n : P.cpb;
+}
+__host__ __device__ inline int wgrad_units(const WgradPlan& P, int chunks) {
+  return chunks > 1 ? 9 : P.kc == 64 ? 5 : 3;
+}
+__host__ __device__ inline int wgrad_block_sets(const WgradPlan& P, int block) {
+  return (wgrad_units(P, wgrad_chunks(P, block)) + P.per - 1) / P.per;
+}
+struct WgradSet {
+  int block, u0, u1;
+};
+__host__ __device__ inline WgradSet wgrad_set(const WgradPlan& P, int set) {
+  WgradSet w;  // every block but the last has as many sets as the first
+  const int f = wgrad_block_sets(P, 0);
+  w.block = set / f < P.blocks - 1 ? set / f : P.blocks - 1;
+  w.u0 = (set - w.block * f) * P.per;
+  const int U = wgrad_units(P, wgrad_chunks(P, w.block));
+  w.u1 = w.u0 + P.per < U ? w.u0 + P.per : U;
+  return w;
+}
+// Tap of a unit's run 0, and whether run 1 is the tap a row below (else it is
+// the next pixel's or, with several chunks, the next chunk's).
+struct WgradUnit {
+  int ky, kx, down;
+};
+__host__ __device__ inline WgradUnit wgrad_unit(const WgradPlan& P, int chunks, int u) {
+  if (chunks > 1) return {u / 3, u % 3, 0};
+  if (P.kc == 32) return {u, 0, 0};
+  return {u < 2 ? 0 : u == 2 ? 1 : 2, u == 1 || u == 4 ? 2 : 0, u == 1};
+}
+// Row m of a unit: its tap and input channel; false: unused.
+__host__ __device__ inline bool wgrad_row(const WgradPlan& P, int block, int u, int m, int* tap,
+                                          int* ci) {
+  const int chunks = wgrad_chunks(P, block), j = m / P.kc;
+  const WgradUnit n = wgrad_unit(P, chunks, u);
+  *ci = block * P.cpb * P.kc + m % P.kc;
+  *tap = 3 * n.ky + n.kx;
+  if (chunks > 1) {
+    *ci += j * P.kc;
+    return j < chunks;
+  }
+  *tap += n.down ? 3 * j : j;
+  return n.down ? j < 2 : n.kx + j < 3 && (P.kc == 32 || j < 2);
+}
 struct WgradArgs {
-  CUtensorMap tin;   // input view {cin, W, H, B}, box {ka, pw, ph, 1}
-  CUtensorMap tdy;   // output-gradient view {cout, W, H, B}, box {kb, pw, ph, 1}
+  CUtensorMap tin;   // input view {cin, W, H, B}, box {kc, q pw + 2, ph, 1}
+  CUtensorMap tdy;   // output-gradient view {cout, W, H, B}, box {kb, q pw, ph, 1}
+  WgradPlan plan;
   int B, H, W;
-  int cin, cout, ka, kb;  // ka, kb: 64 or 32 channels per box
-  int pw, ph;             // pixel box: pw x ph = 64
-  int mtiles, splits, stages;
-  float* partial;         // [splits][mtiles * 128][cout]
+  int cin, cout;
+  float* partial;    // [split][set][per][cout][128]
   int* status;
 };
 
-void launch_conv(const ConvArgs& a, cudaStream_t st);
+int launch_conv(ConvArgs a, cudaStream_t st);  // chooses n, ns, stages; SWEEP_OK or an error
+WgradPlan wgrad_plan(int B, int H, int W, int cin, int cout, size_t* partial);
 void launch_wgrad(const WgradArgs& a, cudaStream_t st);
-size_t conv_smem_bytes(int cout, int kc, int stages);
-size_t wgrad_smem_bytes(int cout, int stages);
 
 // ---- element-wise and reduction kernels (unet_ops.cu)
 struct WeightPrep {  // one 3 x 3 layer of the flat parameter vector
@@ -93,12 +161,12 @@ void launch_head_forward(const bf16* x, const float* theta_head, float* out, lon
 void launch_head_backward(const bf16* x, const float* theta_head, const float* out,
                           const float* target, long long npix, bf16* dpre, double* partial,
                           int nblocks, double* loss, float* grad_head, cudaStream_t st);
-// db[co] = sum_p dy[p][co] (FP32, fixed order)
+// partial[block][co] = sum over the block's pixels of dy[p][co]
 void launch_bias_grad(const bf16* dy, int dy_ps, int cout, long long npix, float* partial,
-                      int nblocks, float* db, cudaStream_t st);
-// dW[co][tap][ci] = sum_s partial[s][tap cin + ci][co]
-void launch_wgrad_reduce(const float* partial, int splits, int rows_padded, int cin, int cout,
-                         float* dW, cudaStream_t st);
+                      int nblocks, cudaStream_t st);
+// dW[co][tap][ci] from a.partial and db[co] (or NULL) from the nb partials bpart
+void launch_wgrad_reduce(const WgradArgs& a, float* dW, const float* bpart, int nb, float* db,
+                         cudaStream_t st);
 void launch_adam(float* theta, const float* grad, float* m, float* v, long long n, int step,
                  float lr, float b1, float b2, float eps, cudaStream_t st);
 

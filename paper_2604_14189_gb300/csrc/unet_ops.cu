@@ -274,6 +274,7 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const bf16* __restrict__
   const long long p1 = p0 + per < npix ? p0 + per : npix;
   float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   if (r < rows)
+#pragma unroll 8
     for (long long p = p0 + r; p < p1; p += rows) {
       float f[8];
       unpack8(ld8(dy + p * ps + 8 * g), f);
@@ -291,55 +292,86 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const bf16* __restrict__
   }
 }
 
-// db[c] = sum_j partial[j][c]: warp w of the block adds the partials
-// j = w, w + 8, ... for 32 channels (one per lane); the 8 warp sums are then
-// added in a fixed order.
-__global__ void __launch_bounds__(256) bias_grad_total_kernel(const float* partial, int nb,
-                                                              int cout, float* db) {
-  __shared__ float red[8][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int c = blockIdx.x * 32 + lane;
-  float t0 = 0.f, t1 = 0.f;
-  int j = w;
-  for (; j + 8 < nb; j += 16) {
-    t0 += partial[(long long)j * cout + c];
-    t1 += partial[(long long)(j + 8) * cout + c];
-  }
-  if (j < nb) t0 += partial[(long long)j * cout + c];
-  red[w][lane] = t0 + t1;
-  __syncthreads();
-  if (w == 0) {
-    float t = 0.f;
-    for (int k = 0; k < 8; ++k) t += red[k][lane];
-    db[c] = t;
-  }
+// dW[co][tap][ci] = sum_s of its partial sums.  A column (set, unit, co) has 128
+// rows, four per lane.  The order is fixed: eight sums of the splits s = w,
+// w + 8, ... (each as its even and odd terms), added in turn; a warp does all
+// eight (G = 1) or, of many splits, one (G = 8).  The blocks past those sum the
+// bias gradient's partials the same way, 32 channels each.
+__device__ __forceinline__ void add4(float4& t, const float4& x) {
+  t.x += x.x;
+  t.y += x.y;
+  t.z += x.z;
+  t.w += x.w;
 }
-
-// dW[co][row] = sum_s partial[s][row][co], row = tap cin + ci.  Block
-// (row, 32 output channels): warp w adds the splits s = w, w + 8, ... with
-// one coalesced 128-byte load per split; the 8 warp sums are added in a
-// fixed order.
-__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* __restrict__ partial,
-                                                           int splits, int rows_pad, int rows,
-                                                           int cout, float* __restrict__ dW) {
-  __shared__ float red[8][32];
+template <int G>
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const __grid_constant__ WgradArgs a,
+                                                           const float* __restrict__ bpart,
+                                                           int nb, float* __restrict__ dW,
+                                                           float* __restrict__ db) {
+  __shared__ float4 red[8][32];
+  const WgradPlan& P = a.plan;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int r = blockIdx.x, c = blockIdx.y * 32 + lane;
-  const float* p = partial + (long long)r * cout + c;
-  const long long stride = (long long)rows_pad * cout;
-  float t0 = 0.f, t1 = 0.f;
-  int s = w;
-  for (; s + 8 < splits; s += 16) {
-    t0 += p[s * stride];
-    t1 += p[(s + 8) * stride];
+  const int blocks = P.sets * P.per * a.cout * G / 8;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  if ((int)blockIdx.x >= blocks) {
+    const int c = ((int)blockIdx.x - blocks) * 32 + lane;
+    float t0 = 0.f, t1 = 0.f;
+    int j = w;
+#pragma unroll 8
+    for (; j + 8 < nb; j += 16) {
+      t0 += bpart[(long long)j * a.cout + c];
+      t1 += bpart[(long long)(j + 8) * a.cout + c];
+    }
+    if (j < nb) t0 += bpart[(long long)j * a.cout + c];
+    red[w][lane].x = t0 + t1;
+    __syncthreads();
+    if (w == 0) {
+      float t = 0.f;
+      for (int k = 0; k < 8; ++k) t += red[k][lane].x;
+      db[c] = t;
+    }
+    return;
   }
-  if (s < splits) t0 += p[s * stride];
-  red[w][lane] = t0 + t1;
-  __syncthreads();
-  if (w == 0) {
-    float t = 0.f;
-    for (int k = 0; k < 8; ++k) t += red[k][lane];
-    dW[(long long)c * rows + r] = t;
+  const int col = G == 8 ? blockIdx.x : blockIdx.x * 8 + w;
+  const int n = col % a.cout, q = col / a.cout;
+  const int u = q % P.per, set = q / P.per;
+  const WgradSet ws = wgrad_set(P, set);
+  if (G == 8 && ws.u0 + u >= ws.u1) return;
+  const size_t stride = (size_t)P.sets * P.per * a.cout * 32;
+  const float4* p = reinterpret_cast<const float4*>(a.partial) +
+                    ((size_t)(set * P.per + u) * a.cout + n) * 32 + lane;
+  auto sum = [&](int first) {
+    float4 t0 = zero, t1 = zero;
+    int s = first;
+#pragma unroll 4
+    for (; s + 8 < P.splits; s += 16) {
+      add4(t0, p[s * stride]);
+      add4(t1, p[(s + 8) * stride]);
+    }
+    if (s < P.splits) add4(t0, p[s * stride]);
+    add4(t0, t1);
+    return t0;
+  };
+  float4 t = zero;
+  if (G == 8) {
+    red[w][lane] = sum(w);
+    __syncthreads();
+    if (w) return;
+    for (int k = 0; k < 8; ++k) add4(t, red[k][lane]);
+  } else if (ws.u0 + u < ws.u1) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) add4(t, sum(k));
+  }
+  int tap, ci;  // (four rows lie in one run)
+  if (ws.u0 + u >= ws.u1 || !wgrad_row(P, ws.block, ws.u0 + u, 4 * lane, &tap, &ci)) return;
+  float* o = dW + ((size_t)n * 9 + tap) * a.cin + ci;
+  if ((reinterpret_cast<uintptr_t>(o) & 15) == 0) {
+    *reinterpret_cast<float4*>(o) = t;
+  } else {
+    o[0] = t.x;
+    o[1] = t.y;
+    o[2] = t.z;
+    o[3] = t.w;
   }
 }
 
@@ -416,17 +448,18 @@ void launch_head_backward(const bf16* x, const float* theta_head, const float* o
 }
 
 void launch_bias_grad(const bf16* dy, int dy_ps, int cout, long long npix, float* partial,
-                      int nblocks, float* db, cudaStream_t st) {
+                      int nblocks, cudaStream_t st) {
   bias_grad_kernel<<<nblocks, 256, 0, st>>>(dy, dy_ps, cout, npix, partial);
-  bias_grad_total_kernel<<<cout / 32, 256, 0, st>>>(partial, nblocks, cout, db);
-  note_launches(2);
+  note_launches(1);
 }
 
-void launch_wgrad_reduce(const float* partial, int splits, int rows_padded, int cin, int cout,
-                         float* dW, cudaStream_t st) {
-  const int rows = 9 * cin;
-  wgrad_reduce_kernel<<<dim3(rows, cout / 32), 256, 0, st>>>(partial, splits, rows_padded, rows,
-                                                             cout, dW);
+void launch_wgrad_reduce(const WgradArgs& a, float* dW, const float* bpart, int nb, float* db,
+                         cudaStream_t st) {
+  const int cols = a.plan.sets * a.plan.per * a.cout, bias = db ? a.cout / 32 : 0;
+  if (a.plan.splits > 32)
+    wgrad_reduce_kernel<8><<<cols + bias, 256, 0, st>>>(a, bpart, nb, dW, db);
+  else
+    wgrad_reduce_kernel<1><<<cols / 8 + bias, 256, 0, st>>>(a, bpart, nb, dW, db);
   note_launches(1);
 }
 
