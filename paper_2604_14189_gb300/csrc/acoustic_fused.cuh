@@ -79,6 +79,15 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(two(-1.f), b, a); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+// a + b as an atomic addition gives it: subnormal operands and sums are zero.
+__device__ __forceinline__ float add_red(float a, float b) {
+  float r;
+  asm("add.rn.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 add_red(float2 a, float2 b) {
+  return make_float2(add_red(a.x, b.x), add_red(a.y, b.y));
+}
 // a x + b y, the second product rounded on its own
 __device__ __forceinline__ float2 lin2(float2 a, float2 x, float2 b, float2 y) {
   return __ffma2_rn(a, x, mul2(b, y));
@@ -353,7 +362,9 @@ __device__ __forceinline__ void fused_fwd_body(const AcFusedArgs& a, FusedFwdSme
       Row<V> e;
       e.load(U, uc);
       // the plain update, then each axis' CPML term added, as the stencil and
-      // CPML kernels do it: the same roundings
+      // CPML kernels do it: the same roundings.  (In a corner those add the two
+      // terms in either order, but nearly always x first: an x thread has one
+      // addition for its 4 cells, a z thread one per row.)
       float2 L[VP], tz[VP], tx[VP];
 #pragma unroll
       for (int i = 0; i < VP; ++i) {
@@ -421,8 +432,8 @@ __device__ __forceinline__ void fused_fwd_body(const AcFusedArgs& a, FusedFwdSme
       }
 #pragma unroll
       for (int i = 0; i < VP; ++i) {
-        if (zs) out.v[i] = add2(out.v[i], tz[i]);
-        if (xs) out.v[i] = add2(out.v[i], tx[i]);
+        if (xs) out.v[i] = add_red(out.v[i], tx[i]);
+        if (zs) out.v[i] = add_red(out.v[i], tz[i]);
       }
       stv<V>(m.u[cur ^ 1] + q.o, out);
       up = uc;
@@ -496,7 +507,7 @@ __device__ __forceinline__ void fused_bwd_body(const AcFusedArgs& a, FusedBwdSme
   const FusedCells<C> q(g, s, oz, ox, a.steps);
   const bool zs = zb && q.in && z_border(g, q.gz);
   const bool zn = zb && q.in && (q.gz < g.P + 4 || q.gz >= g.P + g.nz - 4);  // zs or next to it
-  const bool xn = xb && q.in && (q.gx < g.P + 4 || q.gx + V - 1 >= g.P + g.nx - 4);
+  const bool xn = xb && q.in && ((q.gx & ~3) < g.P + 4 || (q.gx | 3) >= g.P + g.nx - 4);
   unsigned zm = 0, xm = 0, im = 0, rm = 0;  // strip rows / columns of the windows, interior, ring
   if (zn)
 #pragma unroll
@@ -784,8 +795,8 @@ __device__ __forceinline__ void fused_bwd_body(const AcFusedArgs& a, FusedBwdSme
         out.v[i] = fma2(kk.v[i], L[i], sub2(add2(mc.v[i], mc.v[i]), mp.v[i]));
 #pragma unroll
       for (int i = 0; i < VP; ++i) {
-        if (zn) out.v[i] = add2(out.v[i], tz[i]);
-        if (xn) out.v[i] = add2(out.v[i], tx[i]);
+        if (xn) out.v[i] = add_red(out.v[i], tx[i]);
+        if (zn) out.v[i] = add_red(out.v[i], tz[i]);
       }
       if (nl > 0) {  // mu^n(r) += K(r) r^{n-1}
         float* I = m.inj[j & 1] + q.o;
@@ -795,7 +806,8 @@ __device__ __forceinline__ void fused_bwd_body(const AcFusedArgs& a, FusedBwdSme
         for (int c = 0; c < V; ++c) any = any || v[c] != 0.f;
         if (any) {
 #pragma unroll
-          for (int i = 0; i < VP; ++i) out.v[i] = add2(out.v[i], mul2(kk.v[i], v.v[i]));
+          for (int c = 0; c < V; ++c)
+            if (v[c] != 0.f) out[c] = add_red(out[c], __fmul_rn(kk[c], v[c]));
           stv<V>(I, zv);
         }
       }
