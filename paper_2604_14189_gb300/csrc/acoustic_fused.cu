@@ -27,22 +27,22 @@ __global__ void __launch_bounds__(C::NT, RES)
 
 struct Variant {
   FusedShape s;
-  int res;                 // CTAs per SM
+  int res, waves;          // CTAs per SM; most waves it is used for
   int threads;
   size_t smem, rec_bytes;  // fixed shared memory, and more per receiver
   void (*kernel)(const AcFusedArgs);
 };
 
-template <int T, int BZ, int BX, int V, int RES>
+template <int T, int BZ, int BX, int V, int RES, int WAVES>
 Variant fwd_variant() {
   using C = FusedTile<T, BZ, BX, V>;
-  return {{T, BZ, BX}, RES, C::NT, sizeof(FusedFwdSmem<C>), sizeof(int2),
+  return {{T, BZ, BX}, RES, WAVES, C::NT, sizeof(FusedFwdSmem<C>), sizeof(int2),
           ac_fused_fwd_kernel<C, RES>};
 }
-template <int T, int BZ, int BX, int V, int RES>
+template <int T, int BZ, int BX, int V, int RES, int WAVES>
 Variant bwd_variant() {
   using C = FusedTile<T, BZ, BX, V>;
-  return {{T, BZ, BX}, RES, C::NT, sizeof(FusedBwdSmem<C>), sizeof(int2) + 4 * T,
+  return {{T, BZ, BX}, RES, WAVES, C::NT, sizeof(FusedBwdSmem<C>), sizeof(int2) + 4 * T,
           ac_fused_bwd_kernel<C, RES>};
 }
 
@@ -60,17 +60,16 @@ Variant bwd_variant() {
 //             2 steps, 32 x 32, one: 5.0 (141 x 187)
 //             1 step, 16 x 32, three: 5.8 | 5.7 | 8.6 | 9.3
 //             1 step, 32 x 32, two: 6.6 | 6.8 | 6.6 | 9.6
-// Past one wave the per-step kernels, which pipeline their loads, are as fast
-// or faster: 301 x 901 + 40 with 20 shots takes them 26.6 us forward against
-// 61, and a second wave of the last forward variant 4.9 to 5.4 us where they
-// take 4.5 to 6.6 (352 x 401 + 29, 2 shots: 4.5 against 4.75).  Whole calls: 200 x 200 + 40 forward, 1000
+// Past one wave (forward: two of the last variant) the per-step kernels,
+// which pipeline their loads, are faster: 301 x 901 + 40 with 20 shots takes
+// them 26.6 us forward against 61.  Whole calls: 200 x 200 + 40 forward, 1000
 // steps, 4.40 -> 1.91 ms; 141 x 187 + 23 gradient, 3 shots, 900 steps, 10.8 ->
 // 6.0 ms.
 const Variant* variants(int dir, int* n) {
-  static const Variant f[] = {fwd_variant<3, 24, 24, 4, 1>(), fwd_variant<2, 32, 32, 4, 1>(),
-                              fwd_variant<2, 24, 24, 4, 2>(), fwd_variant<2, 24, 24, 4, 3>()};
-  static const Variant b[] = {bwd_variant<2, 24, 24, 2, 1>(), bwd_variant<2, 32, 32, 4, 1>(),
-                              bwd_variant<1, 16, 32, 4, 3>(), bwd_variant<1, 32, 32, 4, 2>()};
+  static const Variant f[] = {fwd_variant<3, 24, 24, 4, 1, 1>(), fwd_variant<2, 32, 32, 4, 1, 1>(),
+                              fwd_variant<2, 24, 24, 4, 2, 1>(), fwd_variant<2, 24, 24, 4, 3, 2>()};
+  static const Variant b[] = {bwd_variant<2, 24, 24, 2, 1, 1>(), bwd_variant<2, 32, 32, 4, 1, 1>(),
+                              bwd_variant<1, 16, 32, 4, 3, 1>(), bwd_variant<1, 32, 32, 4, 2, 1>()};
   *n = dir ? (int)(sizeof(b) / sizeof(b[0])) : (int)(sizeof(f) / sizeof(f[0]));
   return dir ? b : f;
 }
@@ -87,7 +86,7 @@ int fused_variant(const Geom& g, int dir) {
   for (int i = 0; i < n; ++i) {
     const long long ctas = (long long)((g.NX + v[i].s.bx - 1) / v[i].s.bx) *
                            ((g.NZ + v[i].s.bz - 1) / v[i].s.bz) * g.nshot;
-    if (ctas <= sms * v[i].res) return i;
+    if (ctas <= sms * v[i].res * v[i].waves) return i;
   }
   return -1;
 }
