@@ -409,7 +409,7 @@ __device__ __forceinline__ void fused_fwd_body(const AcFusedArgs& a, FusedFwdSme
           const float2 d2u = e.d2(i), dp = p.d1(i);
           // zero off the strip (a = b = 0)
           zx.v[i] = lin2(A.v[i], zx.v[i], B.v[i], add2(d2u, dp));
-          px.v[i] = lin2(B.v[i], e.d1(i), A.v[i], px.v[i]);
+          px.v[i] = lin2(A.v[i], px.v[i], B.v[i], e.d1(i));
           tx[i] = mul2(kk.v[i], add2(dp, zx.v[i]));
           if (!((xm >> (2 * i)) & 1u)) tx[i].x = 0.f;
           if (!((xm >> (2 * i + 1)) & 1u)) tx[i].y = 0.f;
