@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(C::NT, RES)
 
 struct Variant {
   FusedShape s;
-  int res, waves;          // CTAs per SM; most waves it is used for
+  int res, waves;          // CTAs per SM; most waves it is used for in a gradient
   int threads;
   size_t smem, rec_bytes;  // fixed shared memory, and more per receiver
   void (*kernel)(const AcFusedArgs);
@@ -60,9 +60,13 @@ Variant bwd_variant() {
 //             2 steps, 32 x 32, one: 5.0 (141 x 187)
 //             1 step, 16 x 32, three: 5.8 | 5.7 | 8.6 | 9.3
 //             1 step, 32 x 32, two: 6.6 | 6.8 | 6.6 | 9.6
-// Past one wave (forward: two of the last variant) the per-step kernels,
-// which pipeline their loads, are faster: 301 x 901 + 40 with 20 shots takes
-// them 26.6 us forward against 61.  Whole calls: 200 x 200 + 40 forward, 1000
+// Past one wave the per-step kernels, which pipeline their loads, are as fast
+// or faster: 301 x 901 + 40 with 20 shots takes them 26.6 us forward against
+// 61.  A second wave of the last forward variant pays where the forward saves
+// its ring (the per-step kernels do that at a cost, these at none): gradients
+// on 36 random grids of 457 to 912 CTAs take 1.0 to 1.3 times as long without
+// it; forward runs alone 0.92 to 1.4 times (352 x 401 + 29, 2 shots: 4.8 us a
+// step against 5.1), so they don't take it.  Whole calls: 200 x 200 + 40 forward, 1000
 // steps, 4.40 -> 1.91 ms; 141 x 187 + 23 gradient, 3 shots, 900 steps, 10.8 ->
 // 6.0 ms.
 const Variant* variants(int dir, int* n) {
@@ -78,7 +82,7 @@ constexpr size_t kMaxSmem = 227 * 1024;
 
 }  // namespace
 
-int fused_variant(const Geom& g, int dir) {
+int fused_variant(const Geom& g, int dir, bool save) {
   if (g.nrec > kFusedMaxRec || g.nshot < 1) return -1;
   int n;
   const Variant* v = variants(dir, &n);
@@ -86,7 +90,8 @@ int fused_variant(const Geom& g, int dir) {
   for (int i = 0; i < n; ++i) {
     const long long ctas = (long long)((g.NX + v[i].s.bx - 1) / v[i].s.bx) *
                            ((g.NZ + v[i].s.bz - 1) / v[i].s.bz) * g.nshot;
-    if (ctas <= sms * v[i].res * v[i].waves) return i;
+    const int waves = save ? v[i].waves : 1;
+    if (ctas <= sms * v[i].res * waves) return i;
   }
   return -1;
 }

@@ -192,12 +192,12 @@ bool deterministic(const sweep_problem* p) {
   return (p->flags & SWEEP_F_DETERMINISTIC) != 0;
 }
 
-// The fused kernels' variant for a problem's forward (dir 0) or backward
-// (dir 1) loop; -1: the stencil and CPML kernels.
-int fused_of(const sweep_problem* p, int dir) {
+// The fused kernels' variant for a problem's forward (dir 0; save: of a
+// gradient, with its ring) or backward (dir 1) loop; -1: the stencil and CPML kernels.
+int fused_of(const sweep_problem* p, int dir, bool save = false) {
   if (p->physics != SWEEP_ACOUSTIC || deterministic(p) || (p->flags & SWEEP_F_ONE_LAUNCH))
     return -1;
-  return fused_variant(make_geom(p), dir);
+  return fused_variant(make_geom(p), dir, save);
 }
 
 Layout layout(const sweep_problem* p, int mode) {
@@ -286,7 +286,7 @@ Layout layout(const sweep_problem* p, int mode) {
     L.graw = b.take(F);
     L.iraw = b.take(F);
   }
-  const bool ff = mode != SWEEP_MODE_ADJOINT && fused_of(p, 0) >= 0;
+  const bool ff = mode != SWEEP_MODE_ADJOINT && fused_of(p, 0, mode == SWEEP_MODE_GRADIENT) >= 0;
   const bool fb = mode != SWEEP_MODE_FORWARD && fused_of(p, 1) >= 0;
   if (ff || (fb && mode == SWEEP_MODE_GRADIENT))
     for (size_t& o : L.u2) o = b.take(F);
@@ -535,7 +535,7 @@ int fused_forward_loop(const sweep_problem* p, const Layout& L, void* ws, int va
 int acoustic_forward_loop(const sweep_problem* p, const Layout& L, void* ws,
                           const float* wavelet, const int32_t* src, const int32_t* rec,
                           float* data, bool save_ring, cudaStream_t st) {
-  if (const int v = fused_of(p, 0); v >= 0)
+  if (const int v = fused_of(p, 0, save_ring); v >= 0)
     return fused_forward_loop(p, L, ws, v, wavelet, src, rec, data, save_ring, st);
   PhaseRange r("sweep acoustic forward");
   AcFwdLoop f;
