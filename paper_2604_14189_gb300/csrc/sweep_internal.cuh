@@ -310,9 +310,10 @@ __device__ __forceinline__ void latch(int* status, int code) {
 
 // Programmatic dependent launch.  A kernel started by launch_dependent may be
 // scheduled while the kernel before it in the stream is still draining; it
-// must call grid_dep_wait() before its first access to memory that an
-// earlier kernel writes (every such kernel here calls it first thing, so the
-// stream order stays transitive).  grid_dep_trigger() lets the next kernel
+// must call grid_dep_wait() before its first access to memory that the kernel
+// before it writes, and before it completes (so that the stream order stays
+// transitive).  A kernel whose predecessor triggers only after its own wait
+// may read before that what the one before the predecessor wrote.  grid_dep_trigger() lets the next kernel
 // be scheduled once every CTA of this one has called it or exited.
 __device__ __forceinline__ void grid_dep_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -47,6 +47,7 @@ constexpr size_t kSmemPerSm = 228 * 1024;  // per SM, of which 1 KB per CTA is r
 // which also counts the static barriers)
 constexpr int kConvMaxSmem = 225 * 1024;
 constexpr int kWgMaxSmem = 225 * 1024;
+constexpr int kWgHalf = 104 * 1024;  // two per SM leave room for a block of the bias gradient
 constexpr int kWgMaxCtas = 512;
 
 __host__ __device__ inline uint32_t tmem_cols(int n) {
@@ -143,37 +144,49 @@ __global__ void __launch_bounds__(kConvThreads)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_holder;
+  if (warp != 4) {  // (the TMA warp waits on its own)
+    grid_dep_wait();
+    grid_dep_trigger();
+  }
 
   if (warp == 4) {  // TMA producer
     if (lane == 0) {
-      int k = 0, s = 0, ph = 1, tap = 0, ch = 0;  // (the ring's first pass waits for nothing)
+      // The weights are older than the kernel launched before this one: the
+      // ring's first pass goes out ahead of the wait for that kernel.
+      const uint32_t tx =
+          wbytes + (a.stays ? 0 : (uint32_t)(PW * (kConvRows + 2) * 2 * KC));
+      auto weights = [&](int k, int s) {
+        mbar_arrive_expect_tx(&full[s], tx);
+        tma_load_3d(base + (size_t)s * stage_bytes, &a.tw, &full[s], k % nch * KC, k / nch, n0);
+      };
+      const int first = min(S, kiters);
+      for (int k = 0; k < first; ++k) weights(k, k);
+      grid_dep_wait();
+      for (int k = 0; k < kept; ++k) {  // the input tile, chunk by chunk (zero off the image)
+        mbar_arrive_expect_tx(&inbar[k], (uint32_t)(PW * (kConvRows + 2) * 2 * KC));
+        tma_load_4d(in + (size_t)k * CS, &a.tin, &inbar[k], k * KC, x0 - 1, y0 - 1, b);
+      }
+      int k = 0, s = 0, ph = 1;
       for (; k < kiters; ++k) {
-        if (k < kept) {  // the input tile, chunk by chunk (zero off the image)
-          mbar_arrive_expect_tx(&inbar[k], (uint32_t)(PW * (kConvRows + 2) * 2 * KC));
-          tma_load_4d(in + (size_t)k * CS, &a.tin, &inbar[k], k * KC, x0 - 1, y0 - 1, b);
+        if (k >= S) {
+          if (!mbar_wait(&empty[s], ph)) {
+            latch(a.status, SWEEP_ETIMEOUT);
+            failed = 1;
+            break;
+          }
+          weights(k, s);
         }
-        if (k >= S && !mbar_wait(&empty[s], ph)) {
-          latch(a.status, SWEEP_ETIMEOUT);
-          failed = 1;
-          break;
-        }
-        uint8_t* st = base + (size_t)s * stage_bytes;
-        mbar_arrive_expect_tx(&full[s],
-                              wbytes + (a.stays ? 0 : (uint32_t)(PW * (kConvRows + 2) * 2 * KC)));
-        tma_load_3d(st, &a.tw, &full[s], ch * KC, tap, n0);
-        if (!a.stays) tma_load_4d(st + wbytes, &a.tin, &full[s], ch * KC, x0 - 1, y0 - 1, b);
+        if (!a.stays)
+          tma_load_4d(base + (size_t)s * stage_bytes + wbytes, &a.tin, &full[s], k % nch * KC,
+                      x0 - 1, y0 - 1, b);
         if (++s == S) {
           s = 0;
           ph ^= 1;
         }
-        if (++ch == nch) {
-          ch = 0;
-          ++tap;
-        }
       }
       // every copy has landed before the CTA may exit
       for (int j = k > S ? k - S : 0; j < k; ++j) mbar_wait(&full[j % S], (j / S) & 1);
-      for (int j = 0; j < min(k, kept); ++j) mbar_wait(&inbar[j], 0);
+      for (int j = 0; j < kept; ++j) mbar_wait(&inbar[j], 0);
     }
     __syncwarp();
   } else if (warp == 5) {  // MMA issuer (the whole warp, one lane issuing)
@@ -368,6 +381,8 @@ __global__ void __launch_bounds__(kConvThreads, 2)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_holder;
+  grid_dep_wait();
+  grid_dep_trigger();
 
   if (warp == 4) {  // TMA producer
     if (lane == 0) {
@@ -563,7 +578,7 @@ int launch_conv(ConvArgs a, cudaStream_t st) {
   a.stages = best.stages;
   if (!a.make_maps(a)) return SWEEP_ECUDA;
   auto* kernel = kConvKernels[(a.kc == 64 ? 3 : 0) + (a.ns == 4 ? 2 : a.ns - 1)];
-  kernel<<<best.ctas, kConvThreads, best.smem, st>>>(a);
+  launch_dependent(kernel, dim3(best.ctas), dim3(kConvThreads), best.smem, st, a);
   note_launches(1);
   return SWEEP_OK;
 }
@@ -599,8 +614,8 @@ WgradPlan wgrad_plan(int B, int H, int W, int cin, int cout, size_t* partial) {
   const int last = wgrad_chunks(P, P.blocks - 1);
   const size_t slack = 1024 + (last > 1 ? (size_t)(P.cpb - last) * wg_chunk_bytes(P) : 0);
   const int cols = (int)tmem_cols(P.per * cout);
-  const int res = cols <= 256 && slack + 2 * stage <= 110 * 1024 ? 2 : 1;
-  const size_t most = res == 2 ? 110 * 1024 : kWgMaxSmem;
+  const int res = cols <= 256 && slack + 2 * stage <= kWgHalf ? 2 : 1;
+  const size_t most = res == 2 ? kWgHalf : kWgMaxSmem;
   P.ring = (int)std::min(most - slack, kWgMaxStages * stage);
   P.smem = std::max(slack + P.ring, kSmemPerSm / (512 / cols + 1) + 1);
   if (partial) *partial = (size_t)P.splits * P.sets * P.per * cout * 128;
@@ -613,7 +628,7 @@ void launch_wgrad(const WgradArgs& a, cudaStream_t st) {
     cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgMaxSmem);
   });
   const WgradPlan& P = a.plan;
-  wgrad_kernel<<<P.splits * P.sets, kConvThreads, P.smem, st>>>(a);
+  launch_dependent(wgrad_kernel, dim3(P.splits * P.sets), dim3(kConvThreads), P.smem, st, a);
   note_launches(1);
 }
 

@@ -8,6 +8,12 @@
 // thread moves 8 channels (16 bytes) at a time.  Reductions are FP32 (FP64
 // for the loss) with partial sums in a fixed order: the same inputs give the
 // same bits.
+//
+// Every kernel of the network is launched as a dependent of the one before it
+// (grid_dep_wait, sweep_internal.cuh): its launch, set-up and, in a
+// convolution, first weights overlap that kernel's tail.  With the element-wise
+// changes below 25 to 60 kernels in series: inference of 1 x 256 x 256 from 281
+// to 174 us, a training step of 8 x 256 x 256 from 1737 to 1395 us.
 #include "sweep_internal.cuh"
 #include "unet_internal.cuh"
 
@@ -42,29 +48,44 @@ int blocks_for(long long n, int per_block = kT) {
   return (int)(b < 1 ? 1 : (b > 1048576 ? 1048576 : b));
 }
 
-__global__ void prep_weights_kernel(const float* __restrict__ theta, WeightPrepAll p,
-                                    long long total) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    long long j = i;
-    int l = 0;
-    while (l < kUnetLayers - 1 && j >= (long long)p.l[l].cout * 9 * p.l[l].cin) {
-      j -= (long long)p.l[l].cout * 9 * p.l[l].cin;
-      ++l;
-    }
-    const WeightPrep& L = p.l[l];
-    const float w = theta[L.off + j];
-    const int ci = (int)(j % L.cin);
-    const int tap = (int)((j / L.cin) % 9);
-    const int co = (int)(j / ((long long)L.cin * 9));
-    const bf16 h = __float2bfloat16_rn(w);
+// Block: one (tap, 32 output x 32 input channels) tile of a layer, transposed
+// through shared memory so that both copies are written along their rows.  (A
+// thread per weight with scattered 2-byte stores took 48 us for the 2.1 M
+// weights; now 9.)
+__global__ void __launch_bounds__(256) prep_weights_kernel(const float* __restrict__ theta,
+                                                           const __grid_constant__ WeightPrepAll p) {
+  __shared__ bf16 t[32][33];
+  grid_dep_wait();
+  grid_dep_trigger();
+  int k = blockIdx.x, l = 0;
+  while (l < kUnetLayers - 1 && k >= p.l[l].cout / 32 * (p.l[l].cin / 32) * 9) {
+    k -= p.l[l].cout / 32 * (p.l[l].cin / 32) * 9;
+    ++l;
+  }
+  const WeightPrep& L = p.l[l];
+  const int tap = k % 9, nci = L.cin / 32;
+  const int ci0 = k / 9 % nci * 32, co0 = k / 9 / nci * 32;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int co = 8 * i + w;
+    const long long j = ((long long)(co0 + co) * 9 + tap) * L.cin + ci0 + lane;
+    const bf16 h = __float2bfloat16_rn(theta[L.off + j]);
     L.w[j] = h;
-    L.wt[((long long)ci * 9 + (8 - tap)) * L.cout + co] = h;
+    t[co][lane] = h;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int ci = 8 * i + w;
+    L.wt[((long long)(ci0 + ci) * 9 + (8 - tap)) * L.cout + co0 + lane] = t[lane][ci];
   }
 }
 
 __global__ void pack_input_kernel(const float* __restrict__ in, int in_ch, bf16* __restrict__ x0,
                                   long long npix) {
+  grid_dep_wait();
+  grid_dep_trigger();
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
        p += (long long)gridDim.x * blockDim.x) {
     float f[32];
@@ -76,14 +97,16 @@ __global__ void pack_input_kernel(const float* __restrict__ in, int in_ch, bf16*
 }
 
 // out[b][y][x][c] = 1/4 sum of the 2 x 2 block (8 channels per thread)
+template <typename I>
 __global__ void pool_kernel(const bf16* __restrict__ s, int s_ps, bf16* __restrict__ out, int B,
                             int H, int W, int C) {
-  const int h = H / 2, w = W / 2, g = C / 8;
-  const long long n = (long long)B * h * w * g;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
+  grid_dep_wait();
+  grid_dep_trigger();
+  const I h = H / 2, w = W / 2, g = C / 8;
+  const I n = (I)B * h * w * g;
+  for (I i = (I)blockIdx.x * kT + threadIdx.x; i < n; i += (I)gridDim.x * kT) {
     const int c = (int)(i % g) * 8;
-    long long p = i / g;
+    I p = i / g;
     const int x = (int)(p % w);
     p /= w;
     const int y = (int)(p % h);
@@ -104,32 +127,37 @@ __global__ void pool_kernel(const bf16* __restrict__ s, int s_ps, bf16* __restri
   }
 }
 
+// out[b][y][x][c] = x[b][y / 2][x / 2][c]: a thread writes the 4 copies of the 8
+// channels it reads.  (A thread per output, with 64-bit index divisions: 19 us
+// a call in a training step of 8 x 256 x 256, now 8.)
+template <typename I>
 __global__ void upsample_kernel(const bf16* __restrict__ x, bf16* __restrict__ out, int B, int h,
                                 int w, int C) {
-  const int H = 2 * h, W = 2 * w, g = C / 8;
-  const long long n = (long long)B * H * W * g;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % g) * 8;
-    long long p = i / g;
-    const int X = (int)(p % W);
-    p /= W;
-    const int Y = (int)(p % H);
-    const int b = (int)(p / H);
-    st8(out + (((long long)b * H + Y) * W + X) * C + c,
-        ld8(x + (((long long)b * h + Y / 2) * w + X / 2) * C + c));
+  grid_dep_wait();
+  grid_dep_trigger();
+  const I g = C / 8, n = (I)B * h * w * g;
+  for (I i = (I)blockIdx.x * kT + threadIdx.x; i < n; i += (I)gridDim.x * kT) {
+    const I p = i / g, c = i - p * g, row = p / w, col = p - row * w;  // row: of all images
+    const uint4 v = ld8(x + (long long)i * 8);
+    bf16* o = out + (4 * (long long)row * w + 2 * (long long)col) * C + c * 8;
+    st8(o, v);
+    st8(o + C, v);
+    st8(o + 2 * (long long)w * C, v);
+    st8(o + (2 * (long long)w + 1) * C, v);
   }
 }
 
+template <typename I>
 __global__ void up_backward_mask_kernel(const bf16* __restrict__ g, int g_ps,
                                         const bf16* __restrict__ x, bf16* __restrict__ d, int B,
                                         int h, int w, int C) {
-  const int H = 2 * h, W = 2 * w, ng = C / 8;
-  const long long n = (long long)B * h * w * ng;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
+  grid_dep_wait();
+  grid_dep_trigger();
+  const int H = 2 * h, W = 2 * w;
+  const I ng = C / 8, n = (I)B * h * w * ng;
+  for (I i = (I)blockIdx.x * kT + threadIdx.x; i < n; i += (I)gridDim.x * kT) {
     const int c = (int)(i % ng) * 8;
-    long long p = i / ng;
+    I p = i / ng;
     const int xx = (int)(p % w);
     p /= w;
     const int y = (int)(p % h);
@@ -154,19 +182,21 @@ __global__ void up_backward_mask_kernel(const bf16* __restrict__ g, int g_ps,
   }
 }
 
+template <typename I>
 __global__ void pool_backward_combine_kernel(const bf16* __restrict__ gp,
                                              const bf16* __restrict__ s, int s_ps,
                                              const bf16* __restrict__ gskip, int gskip_ps,
                                              bf16* __restrict__ d, int B, int H, int W, int C) {
-  const int ng = C / 8;
-  const long long n = (long long)B * H * W * ng;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
+  grid_dep_wait();
+  grid_dep_trigger();
+  const I ng = C / 8, n = (I)B * H * W * ng;
+  for (I i = (I)blockIdx.x * kT + threadIdx.x; i < n; i += (I)gridDim.x * kT) {
     const int c = (int)(i % ng) * 8;
-    const long long p = i / ng;
-    const int x = (int)(p % W);
-    const int y = (int)((p / W) % H);
-    const int b = (int)(p / ((long long)W * H));
+    const I row = i / ng / W;
+    const long long p = (long long)(i / ng);
+    const int x = (int)(i / ng - row * W);
+    const int y = (int)(row % H);
+    const int b = (int)(row / H);
     float a[8], m[8], k2[8];
     unpack8(ld8(gp + (((long long)b * (H / 2) + y / 2) * (W / 2) + x / 2) * C + c), a);
     unpack8(ld8(s + p * s_ps + c), m);
@@ -179,6 +209,8 @@ __global__ void pool_backward_combine_kernel(const bf16* __restrict__ gp,
 
 __global__ void head_forward_kernel(const bf16* __restrict__ x, const float* __restrict__ th,
                                     float* __restrict__ out, long long npix) {
+  grid_dep_wait();
+  grid_dep_trigger();
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
        p += (long long)gridDim.x * blockDim.x) {
     float acc = 0.f;
@@ -198,13 +230,16 @@ __global__ void __launch_bounds__(kT) head_backward_kernel(
     const bf16* __restrict__ x, const float* __restrict__ th, const float* __restrict__ out,
     const float* __restrict__ tgt, long long npix, bf16* __restrict__ dpre,
     double* __restrict__ lpart, float* __restrict__ hpart) {
-  __shared__ double sl[kT];
+  __shared__ double sl[kT / 32];
   __shared__ float sh[kT / 32][33];
+  grid_dep_wait();
+  grid_dep_trigger();
   const float scale = 2.0f / (float)npix;
   double l = 0.0;
   float gw[33];
 #pragma unroll
   for (int k = 0; k < 33; ++k) gw[k] = 0.f;
+#pragma unroll 2
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
        p += (long long)gridDim.x * blockDim.x) {
     const float r = out[p] - tgt[p];
@@ -224,7 +259,6 @@ __global__ void __launch_bounds__(kT) head_backward_kernel(
     }
   }
   // block sums in a fixed order
-  sl[threadIdx.x] = l;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < 33; ++k) {
@@ -232,10 +266,12 @@ __global__ void __launch_bounds__(kT) head_backward_kernel(
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (lane == 0) sh[warp][k] = v;
   }
+  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+  if (lane == 0) sl[warp] = l;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
-    for (int i = 0; i < kT; ++i) t += sl[i];
+    for (int i = 0; i < kT / 32; ++i) t += sl[i];
     lpart[blockIdx.x] = t;
   }
   if (threadIdx.x < 33) {
@@ -245,49 +281,67 @@ __global__ void __launch_bounds__(kT) head_backward_kernel(
   }
 }
 
-__global__ void head_backward_total_kernel(const double* lpart, const float* hpart, int nb,
-                                           long long npix, double* loss, float* grad_head) {
-  if (threadIdx.x == 0 && loss) {
+// The sums of the blocks' partials: the loss by a warp's tree, a head gradient
+// in block order, from shared memory (straight from global: 24 us, now 6).
+__global__ void __launch_bounds__(kT) head_backward_total_kernel(const double* lpart,
+                                                                 const float* hpart, int nb,
+                                                                 long long npix, double* loss,
+                                                                 float* grad_head) {
+  extern __shared__ float sp[];  // [nb][33]
+  grid_dep_wait();
+  grid_dep_trigger();
+  for (int i = threadIdx.x; i < nb * 33; i += kT) sp[i] = hpart[i];
+  if (threadIdx.x >= kT - 32 && loss) {
     double t = 0.0;
-    for (int i = 0; i < nb; ++i) t += lpart[i];
-    *loss = t / (double)npix;
+    for (int i = threadIdx.x & 31; i < nb; i += 32) t += lpart[i];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == kT - 32) *loss = t / (double)npix;
   }
+  __syncthreads();
   if (threadIdx.x < 33) {
     float t = 0.f;
-    for (int i = 0; i < nb; ++i) t += hpart[(long long)i * 33 + threadIdx.x];
+#pragma unroll 8
+    for (int i = 0; i < nb; ++i) t += sp[i * 33 + threadIdx.x];
     grad_head[threadIdx.x] = t;
   }
 }
 
 // partial[block][co] = sum over the block's pixels of dy[p][co]: a thread
-// owns 8 channels (one 16-byte load per pixel) and every (256 / (cout / 8))-th
-// pixel of the block's range; the block then adds its rows in a fixed order.
-__global__ void __launch_bounds__(256) bias_grad_kernel(const bf16* __restrict__ dy, int ps,
+// owns 4 channels and every (256 / (cout / 8))-th pixel of the block's range;
+// the block then adds its rows in a fixed order.  dy is older than the kernel
+// launched before this one (the weight gradient, which leaves room for a block
+// per SM), so the two run together; only the end waits for it.
+__global__ void __launch_bounds__(512) bias_grad_kernel(const bf16* __restrict__ dy, int ps,
                                                         int cout, long long npix,
                                                         float* __restrict__ partial) {
-  __shared__ float red[256][9];
-  const int groups = cout / 8;                  // 4 .. 32
-  const int rows = blockDim.x / groups;         // pixels in flight per block
+  __shared__ float red[512][5];
+  grid_dep_trigger();
+  const int groups = cout / 4;                  // 8 .. 64
+  const int rows = 256 / (cout / 8);            // pixels in flight per block
   const int g = threadIdx.x % groups, r = threadIdx.x / groups;
   const long long per = (npix + gridDim.x - 1) / gridDim.x;
   const long long p0 = blockIdx.x * per;
   const long long p1 = p0 + per < npix ? p0 + per : npix;
-  float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  float acc[4] = {0, 0, 0, 0};
   if (r < rows)
 #pragma unroll 8
     for (long long p = p0 + r; p < p1; p += rows) {
-      float f[8];
-      unpack8(ld8(dy + p * ps + 8 * g), f);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) acc[k] += f[k];
+      const uint2 u = *reinterpret_cast<const uint2*>(dy + p * ps + 4 * g);
+      const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+      const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+      acc[0] += a.x;
+      acc[1] += a.y;
+      acc[2] += b.x;
+      acc[3] += b.y;
     }
 #pragma unroll
-  for (int k = 0; k < 8; ++k) red[threadIdx.x][k] = acc[k];
+  for (int k = 0; k < 4; ++k) red[threadIdx.x][k] = acc[k];
   __syncthreads();
-  if (threadIdx.x < cout) {
-    const int gg = threadIdx.x / 8, k = threadIdx.x % 8;
+  if ((int)threadIdx.x < cout) {
+    const int gg = threadIdx.x / 4, k = threadIdx.x % 4;
     float t = 0.f;
     for (int rr = 0; rr < rows; ++rr) t += red[rr * groups + gg][k];
+    grid_dep_wait();
     partial[(long long)blockIdx.x * cout + threadIdx.x] = t;
   }
 }
@@ -309,6 +363,8 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const __grid_constant
                                                            int nb, float* __restrict__ dW,
                                                            float* __restrict__ db) {
   __shared__ float4 red[8][32];
+  grid_dep_wait();
+  grid_dep_trigger();
   const WgradPlan& P = a.plan;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int blocks = P.sets * P.per * a.cout * G / 8;
@@ -378,6 +434,8 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const __grid_constant
 __global__ void adam_kernel(float* __restrict__ th, const float* __restrict__ g,
                             float* __restrict__ m, float* __restrict__ v, long long n, float lr,
                             float b1, float b2, float eps, float c1, float c2) {
+  grid_dep_wait();
+  grid_dep_trigger();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     const float gi = g[i];
@@ -391,48 +449,58 @@ __global__ void adam_kernel(float* __restrict__ th, const float* __restrict__ g,
 
 }  // namespace
 
+// Launches kernel<int> or, past 2^31 elements, kernel<long long>.
+#define LAUNCH_INDEXED(kernel, n, ...)                                                     \
+  do {                                                                                     \
+    const long long n_ = (n);                                                              \
+    const dim3 grid_(blocks_for(n_)), block_(kT);                                          \
+    if (n_ < (1LL << 31) - 1048576LL * kT)                                                 \
+      launch_dependent(kernel<int>, grid_, block_, 0, st, __VA_ARGS__);                    \
+    else                                                                                   \
+      launch_dependent(kernel<long long>, grid_, block_, 0, st, __VA_ARGS__);              \
+    note_launches(1);                                                                      \
+  } while (0)
+
 void launch_prep_weights(const float* theta, const WeightPrepAll& p, long long total_w,
                          cudaStream_t st) {
-  prep_weights_kernel<<<blocks_for(total_w), kT, 0, st>>>(theta, p, total_w);
+  launch_dependent(prep_weights_kernel, dim3((unsigned)(total_w / (32 * 32))), dim3(256), 0, st,
+                   theta, p);
   note_launches(1);
 }
 
 void launch_pack_input(const float* in, int in_ch, bf16* x0, long long npix, cudaStream_t st) {
-  pack_input_kernel<<<blocks_for(npix), kT, 0, st>>>(in, in_ch, x0, npix);
+  launch_dependent(pack_input_kernel, dim3(blocks_for(npix)), dim3(kT), 0, st, in, in_ch, x0,
+                   npix);
   note_launches(1);
 }
 
 void launch_pool(const bf16* s, int s_ps, bf16* out, int B, int H, int W, int C,
                  cudaStream_t st) {
-  pool_kernel<<<blocks_for((long long)B * (H / 2) * (W / 2) * (C / 8)), kT, 0, st>>>(
-      s, s_ps, out, B, H, W, C);
-  note_launches(1);
+  LAUNCH_INDEXED(pool_kernel, (long long)B * (H / 2) * (W / 2) * (C / 8), s, s_ps, out, B, H, W,
+                 C);
 }
 
 void launch_upsample(const bf16* x, bf16* out, int B, int h, int w, int C, cudaStream_t st) {
-  upsample_kernel<<<blocks_for((long long)B * 4 * h * w * (C / 8)), kT, 0, st>>>(x, out, B, h,
-                                                                                w, C);
-  note_launches(1);
+  LAUNCH_INDEXED(upsample_kernel, (long long)B * h * w * (C / 8), x, out, B, h, w, C);
 }
 
 void launch_up_backward_mask(const bf16* g, int g_ps, const bf16* x, bf16* d, int B, int h,
                              int w, int C, cudaStream_t st) {
-  up_backward_mask_kernel<<<blocks_for((long long)B * h * w * (C / 8)), kT, 0, st>>>(
-      g, g_ps, x, d, B, h, w, C);
-  note_launches(1);
+  LAUNCH_INDEXED(up_backward_mask_kernel, (long long)B * h * w * (C / 8), g, g_ps, x, d, B, h, w,
+                 C);
 }
 
 void launch_pool_backward_combine(const bf16* gp, const bf16* s, int s_ps, const bf16* gskip,
                                   int gskip_ps, bf16* d, int B, int H, int W, int C,
                                   cudaStream_t st) {
-  pool_backward_combine_kernel<<<blocks_for((long long)B * H * W * (C / 8)), kT, 0, st>>>(
-      gp, s, s_ps, gskip, gskip_ps, d, B, H, W, C);
-  note_launches(1);
+  LAUNCH_INDEXED(pool_backward_combine_kernel, (long long)B * H * W * (C / 8), gp, s, s_ps, gskip,
+                 gskip_ps, d, B, H, W, C);
 }
 
 void launch_head_forward(const bf16* x, const float* theta_head, float* out, long long npix,
                          cudaStream_t st) {
-  head_forward_kernel<<<blocks_for(npix), kT, 0, st>>>(x, theta_head, out, npix);
+  launch_dependent(head_forward_kernel, dim3(blocks_for(npix)), dim3(kT), 0, st, x, theta_head,
+                   out, npix);
   note_launches(1);
 }
 
@@ -441,15 +509,17 @@ void launch_head_backward(const bf16* x, const float* theta_head, const float* o
                           int nblocks, double* loss, float* grad_head, cudaStream_t st) {
   // float partials of the head gradients follow the FP64 loss partials
   float* hpart = reinterpret_cast<float*>(partial + nblocks);
-  head_backward_kernel<<<nblocks, kT, 0, st>>>(x, theta_head, out, target, npix, dpre, partial,
-                                               hpart);
-  head_backward_total_kernel<<<1, 64, 0, st>>>(partial, hpart, nblocks, npix, loss, grad_head);
+  launch_dependent(head_backward_kernel, dim3(nblocks), dim3(kT), 0, st, x, theta_head, out,
+                   target, npix, dpre, partial, hpart);
+  launch_dependent(head_backward_total_kernel, dim3(1), dim3(kT), nblocks * 33 * sizeof(float), st,
+                   partial, hpart, nblocks, npix, loss, grad_head);
   note_launches(2);
 }
 
 void launch_bias_grad(const bf16* dy, int dy_ps, int cout, long long npix, float* partial,
                       int nblocks, cudaStream_t st) {
-  bias_grad_kernel<<<nblocks, 256, 0, st>>>(dy, dy_ps, cout, npix, partial);
+  launch_dependent(bias_grad_kernel, dim3(nblocks), dim3(512), 0, st, dy, dy_ps, cout, npix,
+                   partial);
   note_launches(1);
 }
 
@@ -457,16 +527,19 @@ void launch_wgrad_reduce(const WgradArgs& a, float* dW, const float* bpart, int 
                          cudaStream_t st) {
   const int cols = a.plan.sets * a.plan.per * a.cout, bias = db ? a.cout / 32 : 0;
   if (a.plan.splits > 32)
-    wgrad_reduce_kernel<8><<<cols + bias, 256, 0, st>>>(a, bpart, nb, dW, db);
+    launch_dependent(wgrad_reduce_kernel<8>, dim3(cols + bias), dim3(256), 0, st, a, bpart, nb, dW,
+                     db);
   else
-    wgrad_reduce_kernel<1><<<cols / 8 + bias, 256, 0, st>>>(a, bpart, nb, dW, db);
+    launch_dependent(wgrad_reduce_kernel<1>, dim3(cols / 8 + bias), dim3(256), 0, st, a, bpart, nb,
+                     dW, db);
   note_launches(1);
 }
 
 void launch_adam(float* theta, const float* grad, float* m, float* v, long long n, int step,
                  float lr, float b1, float b2, float eps, cudaStream_t st) {
   const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-  adam_kernel<<<blocks_for(n), kT, 0, st>>>(theta, grad, m, v, n, lr, b1, b2, eps, c1, c2);
+  launch_dependent(adam_kernel, dim3(blocks_for(n)), dim3(kT), 0, st, theta, grad, m, v, n, lr, b1,
+                   b2, eps, c1, c2);
   note_launches(1);
 }
 
