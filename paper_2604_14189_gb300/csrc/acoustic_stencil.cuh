@@ -19,7 +19,8 @@ namespace sweep {
 namespace {
 
 
-constexpr int FWD_THREADS = 256;
+constexpr int FWD_THREADS = 256;  // of a group: 8 warps, a tile
+constexpr int FWD_GROUPS = 2;     // most groups of a per-step kernel's CTA
 constexpr int BWD_ROLE_WARPS = 8;  // backward: 8 adjoint + 8 imaging warps
 constexpr int BWD_THREADS = 64 * BWD_ROLE_WARPS;
 
@@ -27,14 +28,14 @@ constexpr int BWD_THREADS = 64 * BWD_ROLE_WARPS;
 // by sweeps on GB300 (301x901+40, 20 shots): forward 32 rows x 4 stages
 // (16 x 6, 32 x 3, 48 x 2, 64 x 2 no better); backward 32 rows x 2 stages,
 // 230 KB of shared memory with the static tables (16 x 3 was 0.5 % slower
-// over the whole gradient).  The 16-row tiles (forward 7 stages, backward
+// over the whole gradient).  The 16-row tiles (forward 6 stages, backward
 // 3) give small grids twice the units.
 template <int BZ>
 struct FwdTile {
   static constexpr int RPW = BZ / (FWD_THREADS / 32);  // rows per warp
   static constexpr int HF = IN_HW * (BZ + 8);          // floats, halo tile
   static constexpr int CF = IN_BX * BZ;                // floats, centre tile
-  static constexpr int STAGES = BZ == IN_BZ ? 4 : 7;
+  static constexpr int STAGES = BZ == IN_BZ ? 4 : 6;
   static constexpr uint32_t BYTES = (HF + 2 * CF) * 4;
   struct __align__(128) Stage {
     float u[HF];   // u^n with halo
@@ -66,12 +67,27 @@ struct BwdTile {
 };
 constexpr size_t kFwdSmem = std::max(FwdTile<IN_BZ>::SMEM, FwdTile<IN_BZ_SMALL>::SMEM);
 constexpr size_t kBwdSmem = std::max(BwdTile<IN_BZ>::SMEM, BwdTile<IN_BZ_SMALL>::SMEM);
-constexpr int kMaxStages = 7;
+constexpr int kMaxStages = 6;
 static_assert(FwdTile<IN_BZ_SMALL>::STAGES <= kMaxStages && BwdTile<IN_BZ_SMALL>::STAGES <= kMaxStages,
               "descriptor ring");
 
 __device__ __forceinline__ float4 lds4(const float* t, int pitch, int r, int c) {
   return *reinterpret_cast<const float4*>(t + r * pitch + c);
+}
+
+// Barrier `id` of a group of N threads; whether any of them passed true.
+template <int N>
+__device__ __forceinline__ bool group_or(int id, bool p) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.s32 p, %1, 0;\n\t"
+      "barrier.cta.red.or.pred q, %2, %3, p;\n\t"
+      "selp.s32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((int)p), "r"(id), "n"(N)
+      : "memory");
+  return r != 0;
 }
 
 struct UnitPos {
@@ -185,6 +201,11 @@ __device__ __forceinline__ bool fwd_body(const AcInFwdArgs& a, const StepCtl& c,
   using C = FwdTile<BZ>;
   using Stage = typename C::Stage;
   constexpr int D = C::STAGES;
+  static_assert(D % FWD_GROUPS == 0, "a stage belongs to one group");
+  // Groups of 8 warps take the CTA's units in turn: one group's barrier, wait
+  // and stores overlap the other's arithmetic (with one, 8 warps an SM issued
+  // an instruction in 34 % of the cycles).
+  const int NG = PDL ? blockDim.x / FWD_THREADS : 1;
   Stage* stg = reinterpret_cast<Stage*>(smem_raw);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + D * sizeof(Stage));
   const Geom& g = a.g;
@@ -196,7 +217,7 @@ __device__ __forceinline__ bool fwd_body(const AcInFwdArgs& a, const StepCtl& c,
   }
   load_shot_table(T, g, a.src, a.wavelet, c.n);
   __syncthreads();  // shot table visible
-  for (int i = threadIdx.x; i < count && i < kUnitTable; i += FWD_THREADS)
+  for (int i = threadIdx.x; i < count && i < kUnitTable; i += NG * FWD_THREADS)
     utab[i] = make_desc(R, g, T, &a, nullptr, c, BZ, bx + i * G);
   if (threadIdx.x == 0) {
     for (int i = 0; i < D; ++i) mbar_init(&bar[i], 1);
@@ -237,15 +258,17 @@ __device__ __forceinline__ bool fwd_body(const AcInFwdArgs& a, const StepCtl& c,
     }
     for (int k = 0; k < D && k < count; ++k) issue(k);
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int grp = PDL ? threadIdx.x / FWD_THREADS : 0;
+  const int tid = threadIdx.x - grp * FWD_THREADS;
+  const int lane = tid & 31, warp = tid >> 5;
   const int lx = 4 * lane, r0 = warp * C::RPW;
-  int k = 0;
-  for (; k < count; ++k) {
+  int k = grp;  // the groups take the units, and so the stages, in turn
+  for (; k < count; k += NG) {
     if constexpr (PDL)
-      if (k == count - 1) grid_dep_trigger();  // the next kernel may start
-    // one CTA barrier per unit: each thread waits for the stage itself, and
-    // the barrier after the unit both releases the stage and agrees on a
-    // transfer that never landed
+      if (k >= count - NG) grid_dep_trigger();  // the next kernel may start
+    // one barrier of the group per unit: each thread waits for the stage
+    // itself, and the barrier after the unit both releases the stage and
+    // agrees on a transfer that never landed
     const bool got = mbar_wait(&bar[k % D], (k / D) & 1);
     const UnitDesc d = k < kUnitTable ? utab[k] : desc[k % D];
     const Stage& sg = stg[k % D];
@@ -290,17 +313,18 @@ __device__ __forceinline__ bool fwd_body(const AcInFwdArgs& a, const StepCtl& c,
       }
     }
     }  // got
-    if (__syncthreads_or(!got)) break;  // stage released
-    if (threadIdx.x == 0 && k + D < count) {
+    if (PDL ? group_or<FWD_THREADS>(1 + grp, !got) : __syncthreads_or(!got))
+      break;  // stage released
+    if (tid == 0 && k + D < count) {
       fence_proxy_async_smem();
       issue(k + D);
     }
   }
   if (k < count) {
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
       // a transfer never landed: report, drain what is still in flight
       latch(a.status, SWEEP_ETIMEOUT);
-      for (int j = k; j < count && j < k + D; ++j) mbar_wait(&bar[j % D], (j / D) & 1);
+      for (int j = k; j < count && j < k + D; j += NG) mbar_wait(&bar[j % D], (j / D) & 1);
     }
     return false;
   }
