@@ -955,6 +955,31 @@ int elastic_reverse_loop(const sweep_problem* p, const Layout& L, void* ws, cons
   return SWEEP_OK;
 }
 
+// One word of page-locked memory, made on first use and freed with its thread;
+// null if there is none.  (Making it must not disturb another thread's capture.)
+class HostWord {
+ public:
+  ~HostWord() {
+    if (p_) cudaFreeHost(p_);
+  }
+  int* get() {
+    if (!p_) {
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      void* p = nullptr;
+      if (cudaHostAlloc(&p, sizeof(int), cudaHostAllocPortable) == cudaSuccess)
+        p_ = static_cast<int*>(p);
+      else
+        cudaGetLastError();
+      cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    return p_;
+  }
+
+ private:
+  int* p_ = nullptr;
+};
+
 }  // namespace
 }  // namespace sweep
 
@@ -1414,12 +1439,16 @@ int sweep_dot(const float* a, const float* b, int64_t n, double* out, void* ws,
 int sweep_status(void* ws, void* stream) {
   if (!ws) return SWEEP_EWORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int h = 0;
-  cudaError_t e = cudaMemcpyAsync(&h, ws, sizeof(int), cudaMemcpyDeviceToHost, st);
+  // Into page-locked memory of this thread: a copy to pageable memory waits for
+  // the stream by itself and goes through a staging buffer.
+  thread_local HostWord word;
+  int local = 0;
+  int* h = word.get() ? word.get() : &local;
+  cudaError_t e = cudaMemcpyAsync(h, ws, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e != cudaSuccess) return SWEEP_ECUDA;
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return SWEEP_ECUDA;
-  return h;
+  return *h;
 }
 
 unsigned long long sweep_kernel_launches(void) { return g_launches.load(); }

@@ -145,7 +145,7 @@ def conv3x3(x, w, bias=None, op=OP_NONE, mask=None, out=None, stream=None):
         _check(mask, torch.bfloat16, (B, H, W, cout), "mask")
     if out is None:
         out = torch.empty((B, H, W, cout), dtype=torch.bfloat16, device=x.device)
-    ws = torch.zeros(256, dtype=torch.uint8, device=x.device)
+    ws = torch.empty(256, dtype=torch.uint8, device=x.device)  # the call clears its status
     rc = _lib.sweep_unet_conv3x3(B, H, W, cin, cout, _ptr(x), _ptr(w), _ptr(bias), int(op),
                                  _ptr(mask), _ptr(out), _ptr(ws), ws.numel(),
                                  sweep._stream(stream))
