@@ -81,16 +81,20 @@ __global__ void el_params_kernel(const ElParamArgs a) {
 // 64 shots): 16 rows x 3 stages x 256 threads 72.0 Gpts/s, 16 x 4 x 256 68.1,
 // 16 x 3 x 512 76.7, 24 x 3 x 256 70.6, 32 x 2 x 256 80.4, 48 x 1 x 256 83.2,
 // 32 x 2 x 512 83.5 (taller tiles read fewer halo rows per output row; 48 and
-// 64 rows spill at 512 threads).  The fields each kernel differentiates (and the coefficients) are
-// staged by a TMA pipeline of E_STAGES stages; the fields it updates in place
-// and the CPML memory variables (read only on tiles that meet a border
-// strip) are read with 16-byte loads issued before the stage wait.
+// 64 rows spill at 512 threads).  The fields each kernel differentiates and those it
+// updates in place are staged by a TMA pipeline of E_STAGES stages; the
+// coefficients, which all shots share and L2 holds, and the CPML memory variables
+// (read only on tiles that meet a border strip) are read with 16-byte loads
+// issued before the stage wait.  Staging the coefficients instead and loading the
+// fields, from DRAM, when their unit began took 715 us a step of 64 shots, this
+// 687 (60 bytes a cell and the strips' memory variables: 6.5 TB/s); prefetching
+// them into L2 a unit ahead 805 (of 8 shots 101, for 106 and 105).
 constexpr int TB_X = 128;
 constexpr int TB_Z = 32;
 constexpr int E_THREADS = 512;
 constexpr int E_RPW = TB_Z / (E_THREADS / 32);  // rows per warp
 constexpr int E_HW = TB_X + 8;                  // x-halo width
-constexpr int E_HZ = TB_Z + 8;                  // z-halo height
+constexpr int E_HZ = TB_Z + 4;                  // z-halo height
 constexpr int E_STAGES = 2;
 constexpr int E_TABLE = 256;                    // unit descriptors per CTA
 
@@ -98,15 +102,15 @@ struct __align__(128) VelStage {
   float txx[TB_Z * E_HW];  // x halo
   float txz[E_HZ * E_HW];  // x and z halos
   float tzz[E_HZ * TB_X];  // z halo
-  float cbx[TB_Z * TB_X];
-  float cbz[TB_Z * TB_X];
+  float vx[TB_Z * TB_X];
+  float vz[TB_Z * TB_X];
 };
 struct __align__(128) StrStage {
   float vx[E_HZ * E_HW];
   float vz[E_HZ * E_HW];
-  float l2m[TB_Z * TB_X];
-  float lam[TB_Z * TB_X];
-  float mu[TB_Z * TB_X];
+  float txx[TB_Z * TB_X];
+  float tzz[TB_Z * TB_X];
+  float txz[TB_Z * TB_X];
 };
 static_assert(sizeof(VelStage) % 128 == 0 && sizeof(StrStage) % 128 == 0, "stage alignment");
 constexpr uint32_t kVelBytes = (TB_Z * E_HW + E_HZ * E_HW + E_HZ * TB_X + 2 * TB_Z * TB_X) * 4;
@@ -222,25 +226,26 @@ __global__ void __launch_bounds__(E_THREADS, 1) el_vel_kernel(const __grid_const
   auto issue = [&](VelStage& sg, uint64_t* b, const EUnit& u) {
     mbar_arrive_expect_tx(b, kVelBytes);
     tma_load_3d(sg.txx, &a.m_txx, b, u.x0 - 4, u.z0, u.s);
-    tma_load_3d(sg.txz, &a.m_txz, b, u.x0 - 4, u.z0 - 4, u.s);
-    tma_load_3d(sg.tzz, &a.m_tzz, b, u.x0, u.z0 - 4, u.s);
-    tma_load_2d(sg.cbx, &a.m_cbx, b, u.x0, u.z0);
-    tma_load_2d(sg.cbz, &a.m_cbz, b, u.x0, u.z0);
+    tma_load_3d(sg.txz, &a.m_txz, b, u.x0 - 4, u.z0 - 2, u.s);
+    tma_load_3d(sg.tzz, &a.m_tzz, b, u.x0, u.z0 - 2, u.s);
+    tma_load_3d(sg.vx, &a.m_vxi, b, u.x0, u.z0, u.s);
+    tma_load_3d(sg.vz, &a.m_vzi, b, u.x0, u.z0, u.s);
   };
   auto body = [&](const EUnit& u, const VelStage& sg, auto wait) {
     const int gx = u.x0 + lx;
     const bool colok = gx < g.NXp;
     const size_t so = (size_t)u.s * g.fstride;
-    // fields updated in place (and memory variables on strip tiles)
-    float vx[E_RPW][4], vz[E_RPW][4], p1[E_RPW][4], p2[E_RPW][4], p3[E_RPW][4], p4[E_RPW][4];
+    // coefficients (and memory variables on strip tiles)
+    float cbx[E_RPW][4], cbz[E_RPW][4], p1[E_RPW][4], p2[E_RPW][4], p3[E_RPW][4], p4[E_RPW][4];
     const bool xs = u.flags & EU_XS, zs = u.flags & EU_ZS;
 #pragma unroll
     for (int q = 0; q < E_RPW; ++q) {
       const int z = u.z0 + r0 + q;
       const bool ok = colok && z < g.NZ;
       const size_t c = so + (size_t)z * g.NXp + gx;
-      f4(ldg4z(a.vx + c, ok), vx[q]);
-      f4(ldg4z(a.vz + c, ok), vz[q]);
+      const size_t m = (size_t)z * g.NXp + gx;
+      f4(ldg4z(a.cbx + m, ok), cbx[q]);
+      f4(ldg4z(a.cbz + m, ok), cbz[q]);
       f4(ldg4z(a.p1 + c, ok && xs), p1[q]);
       f4(ldg4z(a.p3 + c, ok && xs), p3[q]);
       f4(ldg4z(a.p2 + c, ok && zs), p2[q]);
@@ -258,16 +263,16 @@ __global__ void __launch_bounds__(E_THREADS, 1) el_vel_kernel(const __grid_const
     for (int q = 0; q < E_RPW; ++q) {
       const int r = r0 + q, z = u.z0 + r;
       if (z >= g.NZ || !colok) continue;
-      float e[12], f[12], t0[4], t1[4], t2[4], t3[4], bxv[4], bzv[4];
+      float e[12], f[12], t0[4], t1[4], t2[4], t3[4], vx[4], vz[4];
       // vx at (z, x+1/2): Dpx txx (half point), Dmz txz (integer point)
       f4(lds4e(sg.txx, E_HW, r, lx), e);
       f4(lds4e(sg.txx, E_HW, r, lx + 4), e + 4);
       f4(lds4e(sg.txx, E_HW, r, lx + 8), e + 8);
-      f4(lds4e(sg.txz, E_HW, r + 2, lx + 4), t0);
-      f4(lds4e(sg.txz, E_HW, r + 3, lx + 4), t1);
-      f4(lds4e(sg.txz, E_HW, r + 4, lx + 4), t2);
-      f4(lds4e(sg.txz, E_HW, r + 5, lx + 4), t3);
-      f4(lds4e(sg.cbx, TB_X, r, lx), bxv);
+      f4(lds4e(sg.txz, E_HW, r, lx + 4), t0);
+      f4(lds4e(sg.txz, E_HW, r + 1, lx + 4), t1);
+      f4(lds4e(sg.txz, E_HW, r + 2, lx + 4), t2);
+      f4(lds4e(sg.txz, E_HW, r + 3, lx + 4), t3);
+      f4(lds4e(sg.vx, TB_X, r, lx), vx);
       float outx[4], outz[4];
       const float azr = zs ? __ldg(a.az + z) : 0.f, bzr = zs ? __ldg(a.bz + z) : 0.f;
       const float azh = zs ? __ldg(a.azh + z) : 0.f, bzh = zs ? __ldg(a.bzh + z) : 0.f;
@@ -283,17 +288,17 @@ __global__ void __launch_bounds__(E_THREADS, 1) el_vel_kernel(const __grid_const
           p2[q][c] = azr * p2[q][c] + bzr * dzt;
           dzt += p2[q][c];
         }
-        outx[c] = vx[q][c] + bxv[c] * (dxt + dzt);
+        outx[c] = vx[c] + cbx[q][c] * (dxt + dzt);
       }
       // vz at (z+1/2, x): Dmx txz (integer point), Dpz tzz (half point)
-      f4(lds4e(sg.txz, E_HW, r + 4, lx), f);
-      f4(lds4e(sg.txz, E_HW, r + 4, lx + 4), f + 4);
-      f4(lds4e(sg.txz, E_HW, r + 4, lx + 8), f + 8);
-      f4(lds4e(sg.tzz, TB_X, r + 3, lx), t0);
-      f4(lds4e(sg.tzz, TB_X, r + 4, lx), t1);
-      f4(lds4e(sg.tzz, TB_X, r + 5, lx), t2);
-      f4(lds4e(sg.tzz, TB_X, r + 6, lx), t3);
-      f4(lds4e(sg.cbz, TB_X, r, lx), bzv);
+      f4(lds4e(sg.txz, E_HW, r + 2, lx), f);
+      f4(lds4e(sg.txz, E_HW, r + 2, lx + 4), f + 4);
+      f4(lds4e(sg.txz, E_HW, r + 2, lx + 8), f + 8);
+      f4(lds4e(sg.tzz, TB_X, r + 1, lx), t0);
+      f4(lds4e(sg.tzz, TB_X, r + 2, lx), t1);
+      f4(lds4e(sg.tzz, TB_X, r + 3, lx), t2);
+      f4(lds4e(sg.tzz, TB_X, r + 4, lx), t3);
+      f4(lds4e(sg.vz, TB_X, r, lx), vz);
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         float dxt = kS1 * (f[c + 4] - f[c + 3]) + kS2 * (f[c + 5] - f[c + 2]);
@@ -306,7 +311,7 @@ __global__ void __launch_bounds__(E_THREADS, 1) el_vel_kernel(const __grid_const
           p4[q][c] = azh * p4[q][c] + bzh * dzt;
           dzt += p4[q][c];
         }
-        outz[c] = vz[q][c] + bzv[c] * (dxt + dzt);
+        outz[c] = vz[c] + cbz[q][c] * (dxt + dzt);
       }
       const size_t ci = so + (size_t)z * g.NXp + gx;
       stg4(a.vx_o + ci, outx);
@@ -337,17 +342,17 @@ __global__ void __launch_bounds__(E_THREADS, 1) el_str_kernel(const __grid_const
   const int lx = 4 * lane, r0 = warp * E_RPW;
   auto issue = [&](StrStage& sg, uint64_t* b, const EUnit& u) {
     mbar_arrive_expect_tx(b, kStrBytes);
-    tma_load_3d(sg.vx, &a.m_vx, b, u.x0 - 4, u.z0 - 4, u.s);
-    tma_load_3d(sg.vz, &a.m_vz, b, u.x0 - 4, u.z0 - 4, u.s);
-    tma_load_2d(sg.l2m, &a.m_l2m, b, u.x0, u.z0);
-    tma_load_2d(sg.lam, &a.m_lam, b, u.x0, u.z0);
-    tma_load_2d(sg.mu, &a.m_mu, b, u.x0, u.z0);
+    tma_load_3d(sg.vx, &a.m_vx, b, u.x0 - 4, u.z0 - 2, u.s);
+    tma_load_3d(sg.vz, &a.m_vz, b, u.x0 - 4, u.z0 - 2, u.s);
+    tma_load_3d(sg.txx, &a.m_txxi, b, u.x0, u.z0, u.s);
+    tma_load_3d(sg.tzz, &a.m_tzzi, b, u.x0, u.z0, u.s);
+    tma_load_3d(sg.txz, &a.m_txzi, b, u.x0, u.z0, u.s);
   };
   auto body = [&](const EUnit& u, const StrStage& sg, auto wait) {
     const int gx = u.x0 + lx;
     const bool colok = gx < g.NXp;
     const size_t so = (size_t)u.s * g.fstride;
-    float txx[E_RPW][4], tzz[E_RPW][4], txz[E_RPW][4];
+    float l2m[E_RPW][4], lam[E_RPW][4], mu[E_RPW][4];
     float p5[E_RPW][4], p6[E_RPW][4], p7[E_RPW][4], p8[E_RPW][4];
     const bool xs = u.flags & EU_XS, zs = u.flags & EU_ZS;
 #pragma unroll
@@ -355,9 +360,10 @@ __global__ void __launch_bounds__(E_THREADS, 1) el_str_kernel(const __grid_const
       const int z = u.z0 + r0 + q;
       const bool ok = colok && z < g.NZ;
       const size_t c = so + (size_t)z * g.NXp + gx;
-      f4(ldg4z(a.txx + c, ok), txx[q]);
-      f4(ldg4z(a.tzz + c, ok), tzz[q]);
-      f4(ldg4z(a.txz + c, ok), txz[q]);
+      const size_t m = (size_t)z * g.NXp + gx;
+      f4(ldg4z(a.cl2m + m, ok), l2m[q]);
+      f4(ldg4z(a.clam + m, ok), lam[q]);
+      f4(ldg4z(a.cmu + m, ok), mu[q]);
       f4(ldg4z(a.p5 + c, ok && xs), p5[q]);
       f4(ldg4z(a.p8 + c, ok && xs), p8[q]);
       f4(ldg4z(a.p6 + c, ok && zs), p6[q]);
@@ -376,22 +382,22 @@ __global__ void __launch_bounds__(E_THREADS, 1) el_str_kernel(const __grid_const
       const int r = r0 + q, z = u.z0 + r;
       if (z >= g.NZ || !colok) continue;
       float e[12], f[12], v0[4], v1[4], v2[4], v3[4], w0[4], w1[4], w2[4], w3[4];
-      float l2m[4], lam[4], mu[4];
-      f4(lds4e(sg.vx, E_HW, r + 4, lx), e);
-      f4(lds4e(sg.vx, E_HW, r + 4, lx + 4), e + 4);
-      f4(lds4e(sg.vx, E_HW, r + 4, lx + 8), e + 8);
-      f4(lds4e(sg.vz, E_HW, r + 4, lx), f);
-      f4(lds4e(sg.vz, E_HW, r + 4, lx + 4), f + 4);
-      f4(lds4e(sg.vz, E_HW, r + 4, lx + 8), f + 8);
-      f4(lds4e(sg.vx, E_HW, r + 3, lx + 4), v0);
-      f4(lds4e(sg.vx, E_HW, r + 5, lx + 4), v2);
-      f4(lds4e(sg.vx, E_HW, r + 6, lx + 4), v3);
-      f4(lds4e(sg.vz, E_HW, r + 2, lx + 4), w0);
-      f4(lds4e(sg.vz, E_HW, r + 3, lx + 4), w1);
-      f4(lds4e(sg.vz, E_HW, r + 5, lx + 4), w3);
-      f4(lds4e(sg.l2m, TB_X, r, lx), l2m);
-      f4(lds4e(sg.lam, TB_X, r, lx), lam);
-      f4(lds4e(sg.mu, TB_X, r, lx), mu);
+      float txx[4], tzz[4], txz[4];
+      f4(lds4e(sg.vx, E_HW, r + 2, lx), e);
+      f4(lds4e(sg.vx, E_HW, r + 2, lx + 4), e + 4);
+      f4(lds4e(sg.vx, E_HW, r + 2, lx + 8), e + 8);
+      f4(lds4e(sg.vz, E_HW, r + 2, lx), f);
+      f4(lds4e(sg.vz, E_HW, r + 2, lx + 4), f + 4);
+      f4(lds4e(sg.vz, E_HW, r + 2, lx + 8), f + 8);
+      f4(lds4e(sg.vx, E_HW, r + 1, lx + 4), v0);
+      f4(lds4e(sg.vx, E_HW, r + 3, lx + 4), v2);
+      f4(lds4e(sg.vx, E_HW, r + 4, lx + 4), v3);
+      f4(lds4e(sg.vz, E_HW, r, lx + 4), w0);
+      f4(lds4e(sg.vz, E_HW, r + 1, lx + 4), w1);
+      f4(lds4e(sg.vz, E_HW, r + 3, lx + 4), w3);
+      f4(lds4e(sg.txx, TB_X, r, lx), txx);
+      f4(lds4e(sg.tzz, TB_X, r, lx), tzz);
+      f4(lds4e(sg.txz, TB_X, r, lx), txz);
       const float azr = zs ? __ldg(a.az + z) : 0.f, bzr = zs ? __ldg(a.bz + z) : 0.f;
       const float azh = zs ? __ldg(a.azh + z) : 0.f, bzh = zs ? __ldg(a.bzh + z) : 0.f;
 #pragma unroll
@@ -412,8 +418,8 @@ __global__ void __launch_bounds__(E_THREADS, 1) el_str_kernel(const __grid_const
           p6[q][c] = azr * p6[q][c] + bzr * ezz;
           ezz += p6[q][c];
         }
-        txx[q][c] += l2m[c] * exx + lam[c] * ezz;
-        tzz[q][c] += lam[c] * exx + l2m[c] * ezz;
+        txx[c] += l2m[q][c] * exx + lam[q][c] * ezz;
+        tzz[c] += lam[q][c] * exx + l2m[q][c] * ezz;
         // shear stress at (z+1/2, x+1/2): Dpz vx, Dpx vz
         float ezx = kS1 * (v2[c] - v1[c]) + kS2 * (v3[c] - v0[c]);
         float exz = kS1 * (f[c + 5] - f[c + 4]) + kS2 * (f[c + 6] - f[c + 3]);
@@ -425,20 +431,20 @@ __global__ void __launch_bounds__(E_THREADS, 1) el_str_kernel(const __grid_const
           p8[q][c] = axh[c] * p8[q][c] + bxh[c] * exz;
           exz += p8[q][c];
         }
-        txz[q][c] += mu[c] * (ezx + exz);
+        txz[c] += mu[q][c] * (ezx + exz);
       }
       if ((u.flags & EU_SRC) && z == u.sz) {
 #pragma unroll
         for (int c = 0; c < 4; ++c)
           if (gx + c == u.sx) {
-            txx[q][c] += u.amp;
-            tzz[q][c] += u.amp;
+            txx[c] += u.amp;
+            tzz[c] += u.amp;
           }
       }
       const size_t ci = so + (size_t)z * g.NXp + gx;
-      stg4(a.txx_o + ci, txx[q]);
-      stg4(a.tzz_o + ci, tzz[q]);
-      stg4(a.txz_o + ci, txz[q]);
+      stg4(a.txx_o + ci, txx);
+      stg4(a.tzz_o + ci, tzz);
+      stg4(a.txz_o + ci, txz);
       if (xs) {
         stg4(a.p5_o + ci, p5[q]);
         stg4(a.p8_o + ci, p8[q]);
@@ -484,13 +490,11 @@ bool el_step_maps(ElStepArgs& a) {
   auto f3 = [&](CUtensorMap* m, const float* base, uint32_t bx, uint32_t bz) {
     return make_tensor_map(m, base, 3, g.NX, g.NZ, S, g.NXp, (uint64_t)g.fstride, bx, bz, 1);
   };
-  auto f2 = [&](CUtensorMap* m, const float* base) {
-    return make_tensor_map(m, base, 2, g.NX, g.NZ, 1, g.NXp, (uint64_t)g.fstride, TB_X, TB_Z, 1);
-  };
   bool ok = f3(&a.m_txx, a.txx, E_HW, TB_Z) && f3(&a.m_txz, a.txz, E_HW, E_HZ) &&
             f3(&a.m_tzz, a.tzz, TB_X, E_HZ) && f3(&a.m_vx, a.vx_o, E_HW, E_HZ) &&
-            f3(&a.m_vz, a.vz_o, E_HW, E_HZ) && f2(&a.m_cbx, a.cbx) && f2(&a.m_cbz, a.cbz) &&
-            f2(&a.m_l2m, a.cl2m) && f2(&a.m_lam, a.clam) && f2(&a.m_mu, a.cmu);
+            f3(&a.m_vz, a.vz_o, E_HW, E_HZ) && f3(&a.m_vxi, a.vx, TB_X, TB_Z) &&
+            f3(&a.m_vzi, a.vz, TB_X, TB_Z) && f3(&a.m_txxi, a.txx, TB_X, TB_Z) &&
+            f3(&a.m_tzzi, a.tzz, TB_X, TB_Z) && f3(&a.m_txzi, a.txz, TB_X, TB_Z);
   a.ntx = (g.NXp + TB_X - 1) / TB_X;
   a.units = a.ntx * ((g.NZ + TB_Z - 1) / TB_Z) * g.nshot;
   return ok;

@@ -45,9 +45,10 @@ struct ElStepArgs {
   int n;
   // TMA descriptors (built by el_step_maps): stress fields before the step
   // with the halos the velocity kernel needs, velocities after it (read by
-  // the stress kernel) with both halos, coefficients
+  // the stress kernel) with both halos, and the tiles of the fields that each
+  // kernel updates
   CUtensorMap m_txx, m_txz, m_tzz, m_vx, m_vz;
-  CUtensorMap m_cbx, m_cbz, m_l2m, m_lam, m_mu;
+  CUtensorMap m_vxi, m_vzi, m_txxi, m_tzzi, m_txzi;
   int units, ntx;  // (tile, shot) units of the persistent kernels
 };
 void launch_el_params(const ElParamArgs& a, cudaStream_t st);
