@@ -313,7 +313,7 @@ __device__ __forceinline__ bool fwd_body(const AcInFwdArgs& a, const StepCtl& c,
       }
     }
     }  // got
-    if (PDL ? group_or<FWD_THREADS>(1 + grp, !got) : __syncthreads_or(!got))
+    if (NG > 1 ? group_or<FWD_THREADS>(1 + grp, !got) : __syncthreads_or(!got))
       break;  // stage released
     if (tid == 0 && k + D < count) {
       fence_proxy_async_smem();
