@@ -104,7 +104,7 @@ UnetLayout layout(const sweep_unet_shape* s, bool training) {
   for (int l = 0; l < kUnetLayers; ++l) {
     const size_t n = (size_t)kLayer[l].cout * 9 * kLayer[l].cin * sizeof(bf16);
     L.w[l] = b.take(n);
-    L.wt[l] = b.take(n);
+    if (training) L.wt[l] = b.take(n);
   }
   L.x0 = act(1, 32); L.a1 = act(1, 32); L.cat1 = act(1, 64); L.U1 = act(1, 64);
   L.da1 = act(1, 32); L.x1 = act(1, 32);
@@ -158,7 +158,8 @@ bool conv_maps(ConvArgs& a) {
 // One convolution on an H x W level: in (cin channels) * w [cout][9][cin].
 int run_conv(int B, int H, int W, const View& in, const bf16* w, int cin, int cout,
              const float* bias, int op, const bf16* mask, int mask_ps, bf16* out, int out_ps,
-             int* status, cudaStream_t st) {
+             int* status, cudaStream_t st, bf16* pool = nullptr, bf16* up = nullptr,
+             const float* head = nullptr, float* head_out = nullptr) {
   ConvArgs a{};
   a.B = B;
   a.H = H;
@@ -172,6 +173,10 @@ int run_conv(int B, int H, int W, const View& in, const bf16* w, int cin, int co
   a.mask_ps = mask_ps;
   a.out = out;
   a.out_ps = out_ps;
+  a.pool = pool;
+  a.up = up;
+  a.head = head;
+  a.head_out = head_out;
   a.status = status;
   a.in = in.p;
   a.in_ps = in.ps;
@@ -215,10 +220,13 @@ struct Net {
   int w(int level) const { return W >> (level - 1); }
   long long npix(int level) const { return (long long)B * h(level) * w(level); }
 
-  int conv(int level, const View& in, int l, int op, const float* theta, bf16* out, int out_ps) {
+  int conv(int level, const View& in, int l, int op, const float* theta, bf16* out, int out_ps,
+           bf16* pool = nullptr, bf16* up = nullptr, const float* head = nullptr,
+           float* head_out = nullptr) {
     return run_conv(B, h(level), w(level), in, p(L.w[l]), kLayer[l].cin, kLayer[l].cout,
                     theta + layer_off(l) + (long long)kLayer[l].cout * 9 * kLayer[l].cin, op,
-                    nullptr, 0, out, out_ps, status, st);
+                    nullptr, 0, out, out_ps, status, st, pool, up, head,
+                    head_out);
   }
   // data gradient of layer l: dpre (cout channels) -> its input's gradient
   int dgrad(int level, const View& dpre, int l, const bf16* mask, int mask_ps, bf16* out,
@@ -247,7 +255,7 @@ int prep(Net& n, const float* theta) {
     wp.l[l].cin = kLayer[l].cin;
     wp.l[l].cout = kLayer[l].cout;
     wp.l[l].w = n.p(n.L.w[l]);
-    wp.l[l].wt = n.p(n.L.wt[l]);
+    wp.l[l].wt = n.L.wt[l] ? n.p(n.L.wt[l]) : nullptr;
   }
   cudaMemsetAsync(n.status, 0, sizeof(int), n.st);
   launch_prep_weights(theta, wp, total_weights(), n.st);
@@ -261,31 +269,31 @@ int forward(Net& n, const float* theta, const float* input, float* output) {
   launch_pack_input(input, n.s->in_ch, n.p(L.x0), n.npix(1), n.st);
   // encoder
   UNET_TRY(n.conv(1, {n.p(L.x0), 32, 32}, ENC1A, kOpRelu, theta, n.p(L.a1), 32));
-  UNET_TRY(n.conv(1, {n.p(L.a1), 32, 32}, ENC1B, kOpRelu, theta, n.p(L.cat1) + 32, 64));
-  launch_pool(n.p(L.cat1) + 32, 64, n.p(L.p1), B, n.h(1), n.w(1), 32, n.st);
+  UNET_TRY(n.conv(1, {n.p(L.a1), 32, 32}, ENC1B, kOpRelu, theta, n.p(L.cat1) + 32, 64,
+                  n.p(L.p1)));
   UNET_TRY(n.conv(2, {n.p(L.p1), 32, 32}, ENC2A, kOpRelu, theta, n.p(L.a2), 64));
-  UNET_TRY(n.conv(2, {n.p(L.a2), 64, 64}, ENC2B, kOpRelu, theta, n.p(L.cat2) + 64, 128));
-  launch_pool(n.p(L.cat2) + 64, 128, n.p(L.p2), B, n.h(2), n.w(2), 64, n.st);
+  UNET_TRY(n.conv(2, {n.p(L.a2), 64, 64}, ENC2B, kOpRelu, theta, n.p(L.cat2) + 64, 128,
+                  n.p(L.p2)));
   UNET_TRY(n.conv(3, {n.p(L.p2), 64, 64}, ENC3A, kOpRelu, theta, n.p(L.a3), 128));
-  UNET_TRY(n.conv(3, {n.p(L.a3), 128, 128}, ENC3B, kOpRelu, theta, n.p(L.cat3) + 128, 256));
-  launch_pool(n.p(L.cat3) + 128, 256, n.p(L.p3), B, n.h(3), n.w(3), 128, n.st);
+  UNET_TRY(n.conv(3, {n.p(L.a3), 128, 128}, ENC3B, kOpRelu, theta, n.p(L.cat3) + 128,
+                  256, n.p(L.p3)));
   // bottleneck
   UNET_TRY(n.conv(4, {n.p(L.p3), 128, 128}, BOTA, kOpRelu, theta, n.p(L.ba), 256));
-  UNET_TRY(n.conv(4, {n.p(L.ba), 256, 256}, BOTB, kOpRelu, theta, n.p(L.bt), 256));
+  UNET_TRY(n.conv(4, {n.p(L.ba), 256, 256}, BOTB, kOpRelu, theta, n.p(L.bt), 256, nullptr,
+                  n.p(L.U3)));
   // decoder
-  launch_upsample(n.p(L.bt), n.p(L.U3), B, n.h(4), n.w(4), 256, n.st);
   UNET_TRY(n.conv(3, {n.p(L.U3), 256, 256}, UP3, kOpRelu, theta, n.p(L.cat3), 256));
   UNET_TRY(n.conv(3, {n.p(L.cat3), 256, 256}, DEC3A, kOpRelu, theta, n.p(L.da3), 128));
-  UNET_TRY(n.conv(3, {n.p(L.da3), 128, 128}, DEC3B, kOpRelu, theta, n.p(L.x3), 128));
-  launch_upsample(n.p(L.x3), n.p(L.U2), B, n.h(3), n.w(3), 128, n.st);
+  UNET_TRY(n.conv(3, {n.p(L.da3), 128, 128}, DEC3B, kOpRelu, theta, n.p(L.x3), 128, nullptr,
+                  n.p(L.U2)));
   UNET_TRY(n.conv(2, {n.p(L.U2), 128, 128}, UP2, kOpRelu, theta, n.p(L.cat2), 128));
   UNET_TRY(n.conv(2, {n.p(L.cat2), 128, 128}, DEC2A, kOpRelu, theta, n.p(L.da2), 64));
-  UNET_TRY(n.conv(2, {n.p(L.da2), 64, 64}, DEC2B, kOpRelu, theta, n.p(L.x2), 64));
-  launch_upsample(n.p(L.x2), n.p(L.U1), B, n.h(2), n.w(2), 64, n.st);
+  UNET_TRY(n.conv(2, {n.p(L.da2), 64, 64}, DEC2B, kOpRelu, theta, n.p(L.x2), 64, nullptr,
+                  n.p(L.U1)));
   UNET_TRY(n.conv(1, {n.p(L.U1), 64, 64}, UP1, kOpRelu, theta, n.p(L.cat1), 64));
   UNET_TRY(n.conv(1, {n.p(L.cat1), 64, 64}, DEC1A, kOpRelu, theta, n.p(L.da1), 32));
-  UNET_TRY(n.conv(1, {n.p(L.da1), 32, 32}, DEC1B, kOpRelu, theta, n.p(L.x1), 32));
-  launch_head_forward(n.p(L.x1), theta + head_off(), output, n.npix(1), n.st);
+  UNET_TRY(n.conv(1, {n.p(L.da1), 32, 32}, DEC1B, kOpRelu, theta, n.p(L.x1), 32, nullptr,
+                  nullptr, theta + head_off(), output));
   return SWEEP_OK;
 }
 

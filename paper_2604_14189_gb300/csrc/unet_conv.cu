@@ -16,6 +16,9 @@
 // through L2: 8 x 256 x 256 pixels, 32 -> 32 channels, 40 us, now 23 (10 us
 // are the bytes at the copy rate); 8 x 64 x 64, 256 -> 128: 76 us, now 22;
 // 8 x 32 x 32, 256 -> 256: 25 us, now 15 (11 us are the chain of MMAs).
+// The epilogue also writes what the next layer reads instead of the output: its
+// 2 x 2 average, its upsampling or the 1 x 1 head's value, from the same
+// registers (as seven kernels of their own: 12 us of an inference of 174).
 //
 // wgrad_kernel: the weight gradient, a split-K GEMM over the pixels (see
 // WgradPlan in unet_internal.cuh).  Both operands are staged pixel-major by TMA,
@@ -77,6 +80,26 @@ __device__ __forceinline__ uint4 mask8(uint4 w, const uint4& m) {
   return w;
 }
 
+__device__ __forceinline__ uint4 shfl_xor4(const uint4& v, int m) {
+  return make_uint4(
+      __shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m),
+      __shfl_xor_sync(0xffffffffu, v.z, m), __shfl_xor_sync(0xffffffffu, v.w, m));
+}
+
+// Averages of 8 BF16 values each, summed in this order.
+__device__ __forceinline__ uint32_t average4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  auto f = [](const uint32_t& u) {
+    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u));
+  };
+  const float2 x = f(a), y = f(b), z = f(c), w = f(d);
+  return pack2((((x.x + y.x) + z.x) + w.x) * 0.25f, (((x.y + y.y) + z.y) + w.y) * 0.25f);
+}
+__device__ __forceinline__ uint4 average4(const uint4& a, const uint4& b, const uint4& c,
+                                          const uint4& d) {
+  return make_uint4(average4(a.x, b.x, c.x, d.x), average4(a.y, b.y, c.y, d.y),
+                    average4(a.z, b.z, c.z, d.z), average4(a.w, b.w, c.w, d.w));
+}
+
 // Convolution tile: 16 rows x 8 ns columns of pixels.  An accumulator takes
 // 128 of them (16 rows x 8 columns): the 8 pixels of a row are one 8-row core
 // matrix of the A operand, and SBO is the row pitch of the staged tile.
@@ -100,6 +123,7 @@ __global__ void __launch_bounds__(kConvThreads)
   __shared__ uint32_t tmem_holder;
   __shared__ int failed;
   __shared__ __align__(16) float bias[256];
+  __shared__ float head[33];
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_u = smem_u32(smem_raw);
   const uint32_t base_u = (raw_u + 1023u) & ~1023u;
@@ -239,7 +263,8 @@ __global__ void __launch_bounds__(kConvThreads)
   // store covers whole sectors.  The bias and the first step's mask are read
   // while the MMAs run, a step's mask while the step before it is stored.
   const int px = lane >> 2, cu = lane & 3, steps = NS * (a.n / 32);
-  const long long pix0 = ((long long)b * a.H + y0 + 4 * warp) * a.W + x0 + px;
+  const long long row0 = (long long)b * a.H + y0 + 4 * warp;
+  const long long pix0 = row0 * a.W + x0 + px;
   uint4 mk[4];
   auto load_mask = [&](int q, int c0) {
 #pragma unroll
@@ -251,6 +276,7 @@ __global__ void __launch_bounds__(kConvThreads)
   if (warp < 4) {
     if (a.bias)
       for (int i = threadIdx.x; i < a.n; i += 128) bias[i] = a.bias[n0 + i];
+    if (a.head && threadIdx.x < 33) head[threadIdx.x] = a.head[threadIdx.x];
     if (a.op == kOpMask) load_mask(0, 0);
   }
   const bool got = mbar_wait(&done, 0);
@@ -276,6 +302,15 @@ __global__ void __launch_bounds__(kConvThreads)
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] = fmaxf(v[i], 0.f);
       }
+      if (a.head) {  // the 1 x 1 head (cout = 32) of the lane's own pixel
+        const int hr = 4 * warp + (lane >> 3);
+        float t = 0.f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+          t = fmaf(__bfloat162float(__float2bfloat16_rn(v[i])), head[i], t);
+        if (y0 + hr < a.H)
+          a.head_out[((long long)b * a.H + y0 + hr) * a.W + x0 + 8 * q + (lane & 7)] = t + head[32];
+      }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         uint4 w;
@@ -286,7 +321,8 @@ __global__ void __launch_bounds__(kConvThreads)
         *reinterpret_cast<uint4*>(xch + lane * 64 + ((u ^ (lane >> 1)) & 3) * 16) = w;
       }
       __syncwarp();
-      bf16* o = a.out + (pix0 + 8 * q) * a.out_ps + n0 + c0 + 8 * cu;
+      const int ch = n0 + c0 + 8 * cu, col = x0 + 8 * q + px;  // the lane's when it stores
+      bf16* o = a.out + (pix0 + 8 * q) * a.out_ps + ch;
       uint4 w[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -303,6 +339,28 @@ __global__ void __launch_bounds__(kConvThreads)
       for (int i = 0; i < 4; ++i)
         if (y0 + 4 * warp + i < a.H)
           *reinterpret_cast<uint4*>(o + (long long)i * a.W * a.out_ps) = w[i];
+      if (a.up) {  // the nearest upsampling: four copies
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (y0 + 4 * warp + i < a.H) {
+            bf16* d = a.up + (4 * (row0 + i) * a.W + 2 * col) * a.cout + ch;
+            const long long pitch = 2LL * a.W * a.cout;
+            *reinterpret_cast<uint4*>(d) = w[i];
+            *reinterpret_cast<uint4*>(d + a.cout) = w[i];
+            *reinterpret_cast<uint4*>(d + pitch) = w[i];
+            *reinterpret_cast<uint4*>(d + pitch + a.cout) = w[i];
+          }
+      }
+      if (a.pool) {  // the 2 x 2 average (even H, W): the odd columns' lanes hand theirs over
+#pragma unroll
+        for (int i = 0; i < 4; i += 2) {
+          const uint4 r0 = shfl_xor4(w[i], 4), r1 = shfl_xor4(w[i + 1], 4);
+          if (!(px & 1) && y0 + 4 * warp + i < a.H)
+            *reinterpret_cast<uint4*>(
+                a.pool + ((row0 + i) / 2 * (a.W / 2) + col / 2) * a.cout + ch) =
+                average4(w[i], r0, w[i + 1], r1);
+        }
+      }
       __syncwarp();
     }
   }

@@ -41,6 +41,10 @@ struct ConvArgs {
   int mask_ps;
   bf16* out;
   int out_ps;
+  bf16* pool;         // [B][H/2][W/2][cout] 2 x 2 averages of the output, or NULL
+  bf16* up;           // [B][2H][2W][cout] its nearest upsampling, or NULL
+  const float* head;  // cout = 32: weights and bias of the 1 x 1 head, or NULL
+  float* head_out;    // [B][H][W]
   int* status;        // latched on a wait that gives up
   // what the launcher makes the maps from once it has chosen n and ns
   const bf16* w;
@@ -134,7 +138,7 @@ struct WeightPrep {  // one 3 x 3 layer of the flat parameter vector
   long long off;     // W[cout][3][3][cin] in the flat FP32 vector
   int cin, cout;
   bf16* w;           // out [cout][9][cin]
-  bf16* wt;          // out [cin][9][cout], taps mirrored (data gradient)
+  bf16* wt;          // out [cin][9][cout], taps mirrored (data gradient), or NULL
 };
 constexpr int kUnetLayers = 17;
 struct WeightPrepAll {
@@ -143,9 +147,6 @@ struct WeightPrepAll {
 void launch_prep_weights(const float* theta, const WeightPrepAll& p, long long total_w,
                          cudaStream_t st);
 void launch_pack_input(const float* in, int in_ch, bf16* x0, long long npix, cudaStream_t st);
-void launch_pool(const bf16* s, int s_ps, bf16* out, int B, int H, int W, int C,
-                 cudaStream_t st);
-void launch_upsample(const bf16* x, bf16* out, int B, int h, int w, int C, cudaStream_t st);
 // d[p][c] = bf16( (sum over the 2 x 2 children of p of g[child][c]) * (x[p][c] > 0) )
 void launch_up_backward_mask(const bf16* g, int g_ps, const bf16* x, bf16* d, int B, int h,
                              int w, int C, cudaStream_t st);
@@ -153,9 +154,6 @@ void launch_up_backward_mask(const bf16* g, int g_ps, const bf16* x, bf16* d, in
 void launch_pool_backward_combine(const bf16* gp, const bf16* s, int s_ps, const bf16* gskip,
                                   int gskip_ps, bf16* d, int B, int H, int W, int C,
                                   cudaStream_t st);
-// out[p] = sum_c x[p][c] wh[c] + bh; with a target also the loss partials
-void launch_head_forward(const bf16* x, const float* theta_head, float* out, long long npix,
-                         cudaStream_t st);
 // loss = mean (out - t)^2 (FP64); dout = 2 (out - t) / N;
 // dpre[p][c] = bf16(dout[p] wh[c] (x[p][c] > 0)); head gradients
 void launch_head_backward(const bf16* x, const float* theta_head, const float* out,

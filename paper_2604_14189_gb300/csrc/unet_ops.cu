@@ -1,8 +1,9 @@
 // Element-wise and reduction kernels of the U-Net preconditioner: weight
-// conversion to BF16 (and the mirrored transpose the data gradient uses),
-// input packing, 2 x 2 average pooling, nearest 2x upsampling and their
-// backward passes fused with the ReLU masks, the 1 x 1 head with the MSE
-// loss, bias and weight-gradient reductions, and the Adam update.
+// conversion to BF16 (and the mirrored transpose the data gradient uses), input
+// packing, the backward passes of the 2 x 2 average pooling, of the nearest 2x
+// upsampling (both with the ReLU masks) and of the 1 x 1 head with the MSE loss
+// (forward, these three are part of the convolution before them,
+// unet_conv.cu), bias and weight-gradient reductions, and the Adam update.
 //
 // BF16 tensors are NHWC with channel counts that are multiples of 8, so a
 // thread moves 8 channels (16 bytes) at a time.  Reductions are FP32 (FP64
@@ -12,8 +13,9 @@
 // Every kernel of the network is launched as a dependent of the one before it
 // (grid_dep_wait, sweep_internal.cuh): its launch, set-up and, in a
 // convolution, first weights overlap that kernel's tail.  With the element-wise
-// changes below 25 to 60 kernels in series: inference of 1 x 256 x 256 from 281
-// to 174 us, a training step of 8 x 256 x 256 from 1737 to 1395 us.
+// changes below: inference of 1 x 256 x 256 from 281 to 174 us, a training step
+// of 8 x 256 x 256 from 1737 to 1395 us (162 and 1379 with the pooling,
+// upsampling and head in the convolutions).
 #include "sweep_internal.cuh"
 #include "unet_internal.cuh"
 
@@ -74,6 +76,7 @@ __global__ void __launch_bounds__(256) prep_weights_kernel(const float* __restri
     L.w[j] = h;
     t[co][lane] = h;
   }
+  if (!L.wt) return;
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -84,8 +87,8 @@ __global__ void __launch_bounds__(256) prep_weights_kernel(const float* __restri
 
 __global__ void pack_input_kernel(const float* __restrict__ in, int in_ch, bf16* __restrict__ x0,
                                   long long npix) {
-  grid_dep_wait();
-  grid_dep_trigger();
+  // runs next to the weight preparation launched before it, of which it needs
+  // nothing; only its end waits
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
        p += (long long)gridDim.x * blockDim.x) {
     float f[32];
@@ -94,57 +97,8 @@ __global__ void pack_input_kernel(const float* __restrict__ in, int in_ch, bf16*
 #pragma unroll
     for (int q = 0; q < 4; ++q) st8(x0 + p * 32 + 8 * q, pack8(f + 8 * q));
   }
-}
-
-// out[b][y][x][c] = 1/4 sum of the 2 x 2 block (8 channels per thread)
-template <typename I>
-__global__ void pool_kernel(const bf16* __restrict__ s, int s_ps, bf16* __restrict__ out, int B,
-                            int H, int W, int C) {
   grid_dep_wait();
   grid_dep_trigger();
-  const I h = H / 2, w = W / 2, g = C / 8;
-  const I n = (I)B * h * w * g;
-  for (I i = (I)blockIdx.x * kT + threadIdx.x; i < n; i += (I)gridDim.x * kT) {
-    const int c = (int)(i % g) * 8;
-    I p = i / g;
-    const int x = (int)(p % w);
-    p /= w;
-    const int y = (int)(p % h);
-    const int b = (int)(p / h);
-    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-    for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-      for (int dx = 0; dx < 2; ++dx) {
-        float f[8];
-        unpack8(ld8(s + (((long long)b * H + 2 * y + dy) * W + 2 * x + dx) * s_ps + c), f);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] += f[k];
-      }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] *= 0.25f;
-    st8(out + (((long long)b * h + y) * w + x) * C + c, pack8(acc));
-  }
-}
-
-// out[b][y][x][c] = x[b][y / 2][x / 2][c]: a thread writes the 4 copies of the 8
-// channels it reads.  (A thread per output, with 64-bit index divisions: 19 us
-// a call in a training step of 8 x 256 x 256, now 8.)
-template <typename I>
-__global__ void upsample_kernel(const bf16* __restrict__ x, bf16* __restrict__ out, int B, int h,
-                                int w, int C) {
-  grid_dep_wait();
-  grid_dep_trigger();
-  const I g = C / 8, n = (I)B * h * w * g;
-  for (I i = (I)blockIdx.x * kT + threadIdx.x; i < n; i += (I)gridDim.x * kT) {
-    const I p = i / g, c = i - p * g, row = p / w, col = p - row * w;  // row: of all images
-    const uint4 v = ld8(x + (long long)i * 8);
-    bf16* o = out + (4 * (long long)row * w + 2 * (long long)col) * C + c * 8;
-    st8(o, v);
-    st8(o + C, v);
-    st8(o + 2 * (long long)w * C, v);
-    st8(o + (2 * (long long)w + 1) * C, v);
-  }
 }
 
 template <typename I>
@@ -204,24 +158,6 @@ __global__ void pool_backward_combine_kernel(const bf16* __restrict__ gp,
 #pragma unroll
     for (int k = 0; k < 8; ++k) a[k] = (m[k] > 0.f ? 0.25f * a[k] : 0.f) + k2[k];
     st8(d + p * C + c, pack8(a));
-  }
-}
-
-__global__ void head_forward_kernel(const bf16* __restrict__ x, const float* __restrict__ th,
-                                    float* __restrict__ out, long long npix) {
-  grid_dep_wait();
-  grid_dep_trigger();
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
-       p += (long long)gridDim.x * blockDim.x) {
-    float acc = 0.f;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      float f[8];
-      unpack8(ld8(x + p * 32 + 8 * q), f);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) acc = fmaf(f[k], th[8 * q + k], acc);
-    }
-    out[p] = acc + th[32];
   }
 }
 
@@ -474,16 +410,6 @@ void launch_pack_input(const float* in, int in_ch, bf16* x0, long long npix, cud
   note_launches(1);
 }
 
-void launch_pool(const bf16* s, int s_ps, bf16* out, int B, int H, int W, int C,
-                 cudaStream_t st) {
-  LAUNCH_INDEXED(pool_kernel, (long long)B * (H / 2) * (W / 2) * (C / 8), s, s_ps, out, B, H, W,
-                 C);
-}
-
-void launch_upsample(const bf16* x, bf16* out, int B, int h, int w, int C, cudaStream_t st) {
-  LAUNCH_INDEXED(upsample_kernel, (long long)B * h * w * (C / 8), x, out, B, h, w, C);
-}
-
 void launch_up_backward_mask(const bf16* g, int g_ps, const bf16* x, bf16* d, int B, int h,
                              int w, int C, cudaStream_t st) {
   LAUNCH_INDEXED(up_backward_mask_kernel, (long long)B * h * w * (C / 8), g, g_ps, x, d, B, h, w,
@@ -495,13 +421,6 @@ void launch_pool_backward_combine(const bf16* gp, const bf16* s, int s_ps, const
                                   cudaStream_t st) {
   LAUNCH_INDEXED(pool_backward_combine_kernel, (long long)B * H * W * (C / 8), gp, s, s_ps, gskip,
                  gskip_ps, d, B, H, W, C);
-}
-
-void launch_head_forward(const bf16* x, const float* theta_head, float* out, long long npix,
-                         cudaStream_t st) {
-  launch_dependent(head_forward_kernel, dim3(blocks_for(npix)), dim3(kT), 0, st, x, theta_head,
-                   out, npix);
-  note_launches(1);
 }
 
 void launch_head_backward(const bf16* x, const float* theta_head, const float* out,
