@@ -22,8 +22,8 @@
 namespace sweep {
 namespace {
 
-template <int NP>
-__global__ void __launch_bounds__(FWD_GROUPS * FWD_THREADS, 1)
+template <int NP, int NG>
+__global__ void __launch_bounds__(NG * FWD_THREADS, 1)
     ac_in_fwd_kernel(const __grid_constant__ StepBatch<AcInFwdArgs, NP> m) {
   int bx, G;  // this CTA's index and the CTA count of its problem
   const AcInFwdArgs& a = m.p[step_problem(m, &bx, &G)];
@@ -33,9 +33,9 @@ __global__ void __launch_bounds__(FWD_GROUPS * FWD_THREADS, 1)
   __shared__ UnitDesc utab[kUnitTable];
   const StepCtl c{a.n, 0, 0, 0};
   if (a.bz == IN_BZ_SMALL)  // uniform over the CTA: one problem per CTA
-    fwd_body<IN_BZ_SMALL, true>(a, c, bx, G, T, desc, utab, smem_raw);
+    fwd_body<IN_BZ_SMALL, true, NG>(a, c, bx, G, T, desc, utab, smem_raw);
   else
-    fwd_body<IN_BZ, true>(a, c, bx, G, T, desc, utab, smem_raw);
+    fwd_body<IN_BZ, true, NG>(a, c, bx, G, T, desc, utab, smem_raw);
 }
 
 template <int NP, bool INJ>
@@ -122,8 +122,10 @@ int device_sms() {
 template <int NP>
 void set_fwd_attr() {
   static const bool attr = [] {  // thread-safe one-time initialisation
-    cudaFuncSetAttribute(ac_in_fwd_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(ac_in_fwd_kernel<NP, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)kFwdSmem);
+    cudaFuncSetAttribute(ac_in_fwd_kernel<NP, FWD_GROUPS>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem);
     return true;
   }();
   (void)attr;
@@ -138,14 +140,14 @@ void set_bwd_attr() {
   (void)attr;
 }
 
-// Threads of a forward CTA: two groups where a CTA has more than about two
+// Groups of a forward CTA: two where a CTA has more than about two
 // units.  us per step with one group and with two (32-row tiles): 256 x 256 + 40,
 // 16 shots (3.5 units a CTA) 11.4, 10.2; 301 x 901 + 40, 4, 8 and 20 shots (2.5,
 // 5, 12.6) 9.1, 8.6; 12.8, 11.3; 26.8, 24.2.  Below, a larger CTA only delays the
 // CPML kernel: 301 x 901 + 40, 2 shots (1.3) 6.5, 7.8.
-int fwd_threads(long long units) {
+int fwd_groups(long long units) {
   const long long ctas = std::max(1LL, std::min<long long>(device_sms(), units));
-  return FWD_THREADS * (4 * units >= 9 * ctas ? FWD_GROUPS : 1);
+  return 4 * units >= 9 * ctas ? FWD_GROUPS : 1;
 }
 
 void launch_ac_in_fwd(const AcInFwdArgs& a, cudaStream_t st) {
@@ -156,7 +158,9 @@ void launch_ac_in_fwd(const AcInFwdArgs& a, cudaStream_t st) {
   StepBatch<AcInFwdArgs, 1> m;
   m.p[0] = a;
   void* tok = profile_begin(SWEEP_K_AC_FWD_IN, st);
-  launch_dependent(ac_in_fwd_kernel<1>, dim3(grid), dim3(fwd_threads(a.units)), kFwdSmem, st, m);
+  const int ng = fwd_groups(a.units);
+  launch_dependent(ng > 1 ? ac_in_fwd_kernel<1, FWD_GROUPS> : ac_in_fwd_kernel<1, 1>, dim3(grid),
+                   dim3(ng * FWD_THREADS), kFwdSmem, st, m);
   profile_end(tok, st);
   note_launches(1);
 }
@@ -215,7 +219,9 @@ void launch_ac_in_fwd_batch(const AcInFwdArgs* a, int np, cudaStream_t st) {
   set_fwd_attr<kStepBatch>();
   long long units = 0;
   for (int i = 0; i < np; ++i) units += std::max(a[i].units, 0);
-  launch_in_batch(ac_in_fwd_kernel<kStepBatch>, a, np, fwd_threads(units), kFwdSmem, st);
+  const int ng = fwd_groups(units);
+  launch_in_batch(ng > 1 ? ac_in_fwd_kernel<kStepBatch, FWD_GROUPS> : ac_in_fwd_kernel<kStepBatch, 1>,
+                  a, np, ng * FWD_THREADS, kFwdSmem, st);
 }
 
 void launch_ac_in_bwd_batch(const AcInBwdArgs* a, int np, cudaStream_t st) {

@@ -194,18 +194,17 @@ __device__ __forceinline__ void release_barriers(uint64_t* bar, int D) {
 // One CTA's units of a forward step, for tiles of BZ rows.  T, desc and
 // utab are the kernel's static shared tables (one set for both heights).
 // Returns false when a transfer never landed (SWEEP_ETIMEOUT latched).
-template <int BZ, bool PDL>
+template <int BZ, bool PDL, int NG = 1>
 __device__ __forceinline__ bool fwd_body(const AcInFwdArgs& a, const StepCtl& c, int bx, int G,
                                          ShotTable& T, UnitDesc* desc, UnitDesc* utab,
                                          unsigned char* smem_raw) {
   using C = FwdTile<BZ>;
   using Stage = typename C::Stage;
   constexpr int D = C::STAGES;
-  static_assert(D % FWD_GROUPS == 0, "a stage belongs to one group");
-  // Groups of 8 warps take the CTA's units in turn: one group's barrier, wait
+  static_assert(D % NG == 0, "a stage belongs to one group");
+  // NG groups of 8 warps take the CTA's units in turn: one group's barrier, wait
   // and stores overlap the other's arithmetic (with one, 8 warps an SM issued
   // an instruction in 34 % of the cycles).
-  const int NG = PDL ? blockDim.x / FWD_THREADS : 1;
   Stage* stg = reinterpret_cast<Stage*>(smem_raw);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + D * sizeof(Stage));
   const Geom& g = a.g;
@@ -258,7 +257,7 @@ __device__ __forceinline__ bool fwd_body(const AcInFwdArgs& a, const StepCtl& c,
     }
     for (int k = 0; k < D && k < count; ++k) issue(k);
   }
-  const int grp = PDL ? threadIdx.x / FWD_THREADS : 0;
+  const int grp = NG > 1 ? threadIdx.x / FWD_THREADS : 0;
   const int tid = threadIdx.x - grp * FWD_THREADS;
   const int lane = tid & 31, warp = tid >> 5;
   const int lx = 4 * lane, r0 = warp * C::RPW;
