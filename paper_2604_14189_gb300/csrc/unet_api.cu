@@ -159,7 +159,7 @@ bool conv_maps(ConvArgs& a) {
 int run_conv(int B, int H, int W, const View& in, const bf16* w, int cin, int cout,
              const float* bias, int op, const bf16* mask, int mask_ps, bf16* out, int out_ps,
              int* status, cudaStream_t st, bf16* pool = nullptr, bf16* up = nullptr,
-             const float* head = nullptr, float* head_out = nullptr) {
+             const float* head = nullptr, float* head_out = nullptr, bool late = false) {
   ConvArgs a{};
   a.B = B;
   a.H = H;
@@ -177,6 +177,7 @@ int run_conv(int B, int H, int W, const View& in, const bf16* w, int cin, int co
   a.up = up;
   a.head = head;
   a.head_out = head_out;
+  a.late = late;
   a.status = status;
   a.in = in.p;
   a.in_ps = in.ps;
@@ -228,11 +229,15 @@ struct Net {
                     nullptr, 0, out, out_ps, status, st, pool, up, head,
                     head_out);
   }
-  // data gradient of layer l: dpre (cout channels) -> its input's gradient
+  // Data gradient of layer l: dpre (cout channels) -> its input's gradient.
+  // Launched right after the layer's weight gradient, whose last kernel, the
+  // reduction, it runs beside: its inputs are older than the weight gradient,
+  // and nothing in between touches its output.
   int dgrad(int level, const View& dpre, int l, const bf16* mask, int mask_ps, bf16* out,
             int out_ps) {
     return run_conv(B, h(level), w(level), dpre, p(L.wt[l]), kLayer[l].cout, kLayer[l].cin,
-                    nullptr, mask ? kOpMask : kOpNone, mask, mask_ps, out, out_ps, status, st);
+                    nullptr, mask ? kOpMask : kOpNone, mask, mask_ps, out, out_ps, status, st,
+                    nullptr, nullptr, nullptr, nullptr, true);
   }
   int wgrad(int level, const View& x, const View& dpre, int l, float* grad) {
     float* dW = grad + layer_off(l);

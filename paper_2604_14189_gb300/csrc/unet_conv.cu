@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kConvThreads)
   tc_fence_after();
   const uint32_t tmem = tmem_holder;
   if (warp != 4) {  // (the TMA warp waits on its own)
-    grid_dep_wait();
+    if (!a.late) grid_dep_wait();
     grid_dep_trigger();
   }
 
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kConvThreads)
       };
       const int first = min(S, kiters);
       for (int k = 0; k < first; ++k) weights(k, k);
-      grid_dep_wait();
+      if (!a.late) grid_dep_wait();
       for (int k = 0; k < kept; ++k) {  // the input tile, chunk by chunk (zero off the image)
         mbar_arrive_expect_tx(&inbar[k], (uint32_t)(PW * (kConvRows + 2) * 2 * KC));
         tma_load_4d(in + (size_t)k * CS, &a.tin, &inbar[k], k * KC, x0 - 1, y0 - 1, b);
@@ -370,6 +370,7 @@ __global__ void __launch_bounds__(kConvThreads)
     tc_fence_after();
     tmem_dealloc(tmem, ncols);
   }
+  if (a.late) grid_dep_wait();
 }
 
 constexpr int kWgMaxUnits = 3;  // of a CTA

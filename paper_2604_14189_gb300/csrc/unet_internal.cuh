@@ -33,6 +33,8 @@ struct ConvArgs {
   int n, ns;          // a CTA's output channels and 8-pixel column groups
   int stages;         // of the ring
   int stays;          // the input tile is staged once (else once per tap)
+  int late;           // reads and overwrites nothing of the kernel launched before: runs
+                      // beside it, and only its end waits for it
   const float* bias;  // [cout] or NULL
   int op;             // ConvOp
   const bf16* in;
