@@ -78,7 +78,15 @@ const Variant* variants(int dir, int* n) {
   return dir ? b : f;
 }
 
-constexpr size_t kMaxSmem = 227 * 1024;
+constexpr size_t kMaxSmem = 227 * 1024;    // of a CTA
+constexpr size_t kSmemPerSm = 228 * 1024;  // of which each CTA takes 1 KB more than it asks for
+
+// Can `ctas` CTAs that list nrec receivers run in `waves` waves?
+bool runs(const Variant& v, int nrec, long long ctas, int waves) {
+  const size_t need = v.smem + v.rec_bytes * nrec;
+  const long long slots = (long long)device_sms() * waves, res = (ctas + slots - 1) / slots;
+  return res <= v.res && need <= kMaxSmem && res * (need + 1024) <= kSmemPerSm;
+}
 
 }  // namespace
 
@@ -86,12 +94,10 @@ int fused_variant(const Geom& g, int dir, bool save) {
   if (g.nrec > kFusedMaxRec || g.nshot < 1) return -1;
   int n;
   const Variant* v = variants(dir, &n);
-  const long long sms = device_sms();
   for (int i = 0; i < n; ++i) {
     const long long ctas = (long long)((g.NX + v[i].s.bx - 1) / v[i].s.bx) *
                            ((g.NZ + v[i].s.bz - 1) / v[i].s.bz) * g.nshot;
-    const int waves = save ? v[i].waves : 1;
-    if (ctas <= sms * v[i].res * waves) return i;
+    if (runs(v[i], g.nrec, ctas, save ? v[i].waves : 1)) return i;
   }
   return -1;
 }
