@@ -2,6 +2,7 @@
 // the rule that chooses one of them, or the per-step stencil + CPML kernels,
 // for a problem.
 #include <algorithm>
+#include <climits>
 
 #include "acoustic_fused.cuh"
 
@@ -27,7 +28,9 @@ __global__ void __launch_bounds__(C::NT, RES)
 
 struct Variant {
   FusedShape s;
-  int res, waves;          // CTAs per SM; most waves it is used for in a gradient
+  int res;                 // CTAs per SM
+  int waves;               // most waves it is used for in a gradient (else one)
+  int alone;               // most tiles of a shot outside of a gradient
   int threads;
   size_t smem, rec_bytes;  // fixed shared memory, and more per receiver
   void (*kernel)(const AcFusedArgs);
@@ -36,13 +39,13 @@ struct Variant {
 template <int T, int BZ, int BX, int V, int RES, int WAVES>
 Variant fwd_variant() {
   using C = FusedTile<T, BZ, BX, V>;
-  return {{T, BZ, BX}, RES, WAVES, C::NT, sizeof(FusedFwdSmem<C>), sizeof(int2),
+  return {{T, BZ, BX}, RES, WAVES, INT_MAX, C::NT, sizeof(FusedFwdSmem<C>), sizeof(int2),
           ac_fused_fwd_kernel<C, RES>};
 }
-template <int T, int BZ, int BX, int V, int RES, int WAVES>
+template <int T, int BZ, int BX, int V, int RES, int ALONE = INT_MAX>
 Variant bwd_variant() {
   using C = FusedTile<T, BZ, BX, V>;
-  return {{T, BZ, BX}, RES, WAVES, C::NT, sizeof(FusedBwdSmem<C>), sizeof(int2) + 4 * T,
+  return {{T, BZ, BX}, RES, 1, ALONE, C::NT, sizeof(FusedBwdSmem<C>), sizeof(int2) + 4 * T,
           ac_fused_bwd_kernel<C, RES>};
 }
 
@@ -66,14 +69,20 @@ Variant bwd_variant() {
 // its ring (the per-step kernels do that at a cost, these at none): gradients
 // on 36 random grids of 457 to 912 CTAs take 1.0 to 1.3 times as long without
 // it; forward runs alone 0.92 to 1.4 times (352 x 401 + 29, 2 shots: 4.8 us a
-// step against 5.1), so they don't take it.  Whole calls: 200 x 200 + 40 forward, 1000
+// step against 5.1), so they don't take it.  The last backward variant, without
+// the imaging that it takes along in a gradient, is faster than the per-step
+// kernels only on shots of a few tiles, whose cells are mostly border.  An adjoint
+// of 300 steps with 30 and 1000 receivers a shot takes, fused against per step, of
+// 4 tiles (72 shots) 1.70 against 2.11 and 2.15 against 2.72 ms, of 9 (32 shots)
+// 1.65 : 1.90 and 1.94 : 2.07, of 70 (4 shots) 1.45 : 1.51 and 1.67 : 1.52, of 255
+// 1.44 : 1.32 and 1.55 : 1.36.  Whole calls: 200 x 200 + 40 forward, 1000
 // steps, 4.40 -> 1.91 ms; 141 x 187 + 23 gradient, 3 shots, 900 steps, 10.8 ->
 // 6.0 ms.
 const Variant* variants(int dir, int* n) {
   static const Variant f[] = {fwd_variant<3, 24, 24, 4, 1, 1>(), fwd_variant<2, 32, 32, 4, 1, 1>(),
                               fwd_variant<2, 24, 24, 4, 2, 1>(), fwd_variant<2, 24, 24, 4, 3, 2>()};
-  static const Variant b[] = {bwd_variant<2, 24, 24, 2, 1, 1>(), bwd_variant<2, 32, 32, 4, 1, 1>(),
-                              bwd_variant<1, 16, 32, 4, 3, 1>(), bwd_variant<1, 32, 32, 4, 2, 1>()};
+  static const Variant b[] = {bwd_variant<2, 24, 24, 2, 1>(), bwd_variant<2, 32, 32, 4, 1>(),
+                              bwd_variant<1, 16, 32, 4, 3>(), bwd_variant<1, 32, 32, 4, 2, 16>()};
   *n = dir ? (int)(sizeof(b) / sizeof(b[0])) : (int)(sizeof(f) / sizeof(f[0]));
   return dir ? b : f;
 }
@@ -90,14 +99,15 @@ bool runs(const Variant& v, int nrec, long long ctas, int waves) {
 
 }  // namespace
 
-int fused_variant(const Geom& g, int dir, bool save) {
+int fused_variant(const Geom& g, int dir, bool gradient) {
   if (g.nrec > kFusedMaxRec || g.nshot < 1) return -1;
   int n;
   const Variant* v = variants(dir, &n);
   for (int i = 0; i < n; ++i) {
-    const long long ctas = (long long)((g.NX + v[i].s.bx - 1) / v[i].s.bx) *
-                           ((g.NZ + v[i].s.bz - 1) / v[i].s.bz) * g.nshot;
-    if (runs(v[i], g.nrec, ctas, save ? v[i].waves : 1)) return i;
+    const long long tiles = (long long)((g.NX + v[i].s.bx - 1) / v[i].s.bx) *
+                            ((g.NZ + v[i].s.bz - 1) / v[i].s.bz);
+    if (!gradient && tiles > v[i].alone) continue;
+    if (runs(v[i], g.nrec, tiles * g.nshot, gradient ? v[i].waves : 1)) return i;
   }
   return -1;
 }

@@ -192,12 +192,12 @@ bool deterministic(const sweep_problem* p) {
   return (p->flags & SWEEP_F_DETERMINISTIC) != 0;
 }
 
-// The fused kernels' variant for a problem's forward (dir 0; save: of a
-// gradient, with its ring) or backward (dir 1) loop; -1: the stencil and CPML kernels.
-int fused_of(const sweep_problem* p, int dir, bool save = false) {
+// The fused kernels' variant for a problem's forward (dir 0) or backward (dir 1)
+// loop, in a gradient or alone; -1: the stencil and CPML kernels.
+int fused_of(const sweep_problem* p, int dir, bool gradient) {
   if (p->physics != SWEEP_ACOUSTIC || deterministic(p) || (p->flags & SWEEP_F_ONE_LAUNCH))
     return -1;
-  return fused_variant(make_geom(p), dir, save);
+  return fused_variant(make_geom(p), dir, gradient);
 }
 
 Layout layout(const sweep_problem* p, int mode) {
@@ -287,7 +287,7 @@ Layout layout(const sweep_problem* p, int mode) {
     L.iraw = b.take(F);
   }
   const bool ff = mode != SWEEP_MODE_ADJOINT && fused_of(p, 0, mode == SWEEP_MODE_GRADIENT) >= 0;
-  const bool fb = mode != SWEEP_MODE_FORWARD && fused_of(p, 1) >= 0;
+  const bool fb = mode != SWEEP_MODE_FORWARD && fused_of(p, 1, mode == SWEEP_MODE_GRADIENT) >= 0;
   if (ff || (fb && mode == SWEEP_MODE_GRADIENT))
     for (size_t& o : L.u2) o = b.take(F);
   if (ff) {  // a gradient's backward buffers are free during its forward loop
@@ -738,7 +738,7 @@ int acoustic_backward_loop(const sweep_problem* p, const Layout& L, void* ws,
                            const float* wavelet, const int32_t* src, const int32_t* rec,
                            const float* res, float* wgrad, bool imaging, bool illum,
                            cudaStream_t st) {
-  if (const int v = fused_of(p, 1); v >= 0)
+  if (const int v = fused_of(p, 1, imaging); v >= 0)
     return fused_backward_loop(p, L, ws, v, wavelet, src, rec, res, wgrad, imaging, illum, st);
   PhaseRange r("sweep acoustic backward");
   AcBwdLoop b;

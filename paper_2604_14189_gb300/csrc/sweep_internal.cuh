@@ -253,9 +253,9 @@ struct FusedShape {
   int T, bz, bx;  // steps per launch, tile rows and columns
 };
 constexpr int kFusedMaxRec = 2048;  // receivers per shot a CTA can list
-// The variant a problem's forward (dir 0) or backward (dir 1) loop runs, or
-// -1: the stencil + CPML kernels are the faster ones.
-int fused_variant(const Geom& g, int dir, bool save);
+// The variant a problem's forward (dir 0) or backward (dir 1) loop runs, in a
+// gradient or alone, or -1: the stencil + CPML kernels are the faster ones.
+int fused_variant(const Geom& g, int dir, bool gradient);
 FusedShape fused_shape(int dir, int variant);
 void launch_ac_fused(int dir, int variant, const AcFusedArgs& a, cudaStream_t st);
 
