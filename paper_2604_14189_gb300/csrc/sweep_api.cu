@@ -956,22 +956,30 @@ int elastic_reverse_loop(const sweep_problem* p, const Layout& L, void* ws, cons
 }
 
 // One word of page-locked memory, made on first use and freed with its thread;
-// null if there is none.  (Making it must not disturb another thread's capture.)
+// null if there is none.  Making and freeing it are calls that would spoil a
+// capture in the global mode by another thread, were this thread not in the
+// relaxed mode meanwhile.
 class HostWord {
+  struct Relaxed {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  };
+
  public:
   ~HostWord() {
-    if (p_) cudaFreeHost(p_);
+    if (!p_) return;
+    const Relaxed r;
+    cudaFreeHost(p_);
   }
   int* get() {
     if (!p_) {
-      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-      cudaThreadExchangeStreamCaptureMode(&mode);
+      const Relaxed r;
       void* p = nullptr;
       if (cudaHostAlloc(&p, sizeof(int), cudaHostAllocPortable) == cudaSuccess)
         p_ = static_cast<int*>(p);
       else
         cudaGetLastError();
-      cudaThreadExchangeStreamCaptureMode(&mode);
     }
     return p_;
   }
