@@ -129,7 +129,9 @@ typedef struct {
 } sweep_problem;
 
 /* Bytes of device workspace a call of `mode` needs for `prob` (0 on invalid
- * input).  The workspace must be 256-byte aligned. */
+ * input).  The workspace must be 256-byte aligned.  The flags do not change the
+ * size; an acoustic workspace is enough for every problem that is no larger in
+ * any of nz, nx, pml, nshot, nrec and nt. */
 size_t sweep_workspace_bytes(const sweep_problem* prob, int mode);
 
 /* Forward modelling (Sec. 2.1 Propagator + Source + Receiver; Eq. 2 or 12).

@@ -129,6 +129,7 @@ struct Layout {
   size_t rtile = 0, rlist = 0;    // receiver lists of the backward stencil units
   size_t fwd_lo = 0, fwd_hi = 0;  // contiguous range of forward fields
   size_t adj_lo = 0, adj_hi = 0;  // contiguous range of adjoint fields
+  int fused[2] = {-1, -1};        // fused kernels' variants, forward and backward; -1: none
   size_t total = 0;
 };
 
@@ -192,13 +193,12 @@ bool deterministic(const sweep_problem* p) {
   return (p->flags & SWEEP_F_DETERMINISTIC) != 0;
 }
 
-// The fused kernels' variant for a problem's forward (dir 0) or backward (dir 1)
-// loop, in a gradient or alone; -1: the stencil and CPML kernels.
-int fused_of(const sweep_problem* p, int dir, bool gradient) {
-  if (p->physics != SWEEP_ACOUSTIC || deterministic(p) || (p->flags & SWEEP_F_ONE_LAUNCH))
-    return -1;
-  return fused_variant(make_geom(p), dir, gradient);
-}
+// Room for the fused kernels' second set of the state at the end of every
+// acoustic workspace: as many fields as they would need, up to this.  (The largest
+// problems they run have 3 CTAs of 24 rows per SM, 32 columns each with the row
+// pitch, and 4 fields; 6 waves and 2 fields in a gradient: 5.6 MB at 152 SMs.)  So the
+// size depends neither on the flags nor on the GPU, and grows with the problem.
+constexpr size_t kFusedState = 6 << 20;
 
 Layout layout(const sweep_problem* p, int mode) {
   const Geom g = make_geom(p);
@@ -286,17 +286,20 @@ Layout layout(const sweep_problem* p, int mode) {
     L.graw = b.take(F);
     L.iraw = b.take(F);
   }
-  const bool ff = mode != SWEEP_MODE_ADJOINT && fused_of(p, 0, mode == SWEEP_MODE_GRADIENT) >= 0;
-  const bool fb = mode != SWEEP_MODE_FORWARD && fused_of(p, 1, mode == SWEEP_MODE_GRADIENT) >= 0;
-  if (ff || (fb && mode == SWEEP_MODE_GRADIENT))
+  const bool grad = mode == SWEEP_MODE_GRADIENT;
+  const size_t second = (mode == SWEEP_MODE_FORWARD ? 4 : 2) * align_up(F);
+  L.total = b.off + std::min(second, kFusedState);
+  if (second > kFusedState || deterministic(p) || (p->flags & SWEEP_F_ONE_LAUNCH)) return L;
+  if (mode != SWEEP_MODE_ADJOINT) L.fused[0] = fused_variant(g, 0, grad);
+  if (mode != SWEEP_MODE_FORWARD) L.fused[1] = fused_variant(g, 1, grad);
+  if (mode != SWEEP_MODE_ADJOINT)
     for (size_t& o : L.u2) o = b.take(F);
-  if (ff) {  // a gradient's backward buffers are free during its forward loop
-    L.zex2 = mode == SWEEP_MODE_GRADIENT ? L.zbx[0] : b.take(F);
-    L.zez2 = mode == SWEEP_MODE_GRADIENT ? L.zbz[0] : b.take(F);
-  }
-  if (fb)  // and psi is free during its backward loop
-    for (int i = 0; i < 2; ++i) L.m2[i] = mode == SWEEP_MODE_GRADIENT ? L.psx[i] : b.take(F);
-  L.total = b.off;
+  // a gradient's backward buffers are free during its forward loop, and psi
+  // during its backward loop
+  L.zex2 = grad ? L.zbx[0] : mode == SWEEP_MODE_FORWARD ? b.take(F) : 0;
+  L.zez2 = grad ? L.zbz[0] : mode == SWEEP_MODE_FORWARD ? b.take(F) : 0;
+  for (int i = 0; i < 2; ++i)
+    L.m2[i] = grad ? L.psx[i] : mode == SWEEP_MODE_ADJOINT ? b.take(F) : 0;
   return L;
 }
 
@@ -484,9 +487,9 @@ AcFusedArgs fused_args(const sweep_problem* p, const Layout& L, void* ws, const 
 // Forward loop through the fused kernels: launch k reads state set k % 2 and
 // writes the other one.  The sets are named so that u^{nt} ends in u[nt % 2]
 // and u^{nt-1} in the other, as acoustic_forward_loop leaves them.
-int fused_forward_loop(const sweep_problem* p, const Layout& L, void* ws, int variant,
-                       const float* wavelet, const int32_t* src, const int32_t* rec, float* data,
-                       bool save_ring, cudaStream_t st) {
+int fused_forward_loop(const sweep_problem* p, const Layout& L, void* ws, const float* wavelet,
+                       const int32_t* src, const int32_t* rec, float* data, bool save_ring,
+                       cudaStream_t st) {
   PhaseRange r("sweep acoustic forward");
   AcFusedArgs a = fused_args(p, L, ws, wavelet, src, rec);
   const Geom& g = a.g;
@@ -496,7 +499,7 @@ int fused_forward_loop(const sweep_problem* p, const Layout& L, void* ws, int va
   cudaMemsetAsync(at<char>(ws, L.zez2), 0, F, st);
   a.data = g.nrec > 0 ? data : nullptr;
   a.save = save_ring ? at<float>(ws, L.save) : nullptr;
-  const int T = fused_shape(0, variant).T;
+  const int T = fused_shape(0, L.fused[0]).T;
   const int last = (g.nt + T - 1) / T % 2, A = g.nt & 1;
   size_t u[2], up[2];
   u[last] = L.u[A];
@@ -525,7 +528,7 @@ int fused_forward_loop(const sweep_problem* p, const Layout& L, void* ws, int va
     a.zzo = at<float>(ws, zz[o]);
     a.zxo = at<float>(ws, zx[o]);
     void* tok = profile_begin(SWEEP_K_AC_FWD, st);
-    launch_ac_fused(0, variant, a, st);
+    launch_ac_fused(0, L.fused[0], a, st);
     profile_end(tok, st);
   }
   profile_end(loop, st);
@@ -535,8 +538,8 @@ int fused_forward_loop(const sweep_problem* p, const Layout& L, void* ws, int va
 int acoustic_forward_loop(const sweep_problem* p, const Layout& L, void* ws,
                           const float* wavelet, const int32_t* src, const int32_t* rec,
                           float* data, bool save_ring, cudaStream_t st) {
-  if (const int v = fused_of(p, 0, save_ring); v >= 0)
-    return fused_forward_loop(p, L, ws, v, wavelet, src, rec, data, save_ring, st);
+  if (L.fused[0] >= 0)
+    return fused_forward_loop(p, L, ws, wavelet, src, rec, data, save_ring, st);
   PhaseRange r("sweep acoustic forward");
   AcFwdLoop f;
   const int rc = f.init(p, L, ws, wavelet, src, rec, data, save_ring, st);
@@ -673,16 +676,15 @@ struct AcBwdLoop {
 
 // Backward loop through the fused kernels, from (u^{nt-1}, u^{nt}) as either
 // forward loop leaves them.
-int fused_backward_loop(const sweep_problem* p, const Layout& L, void* ws, int variant,
-                        const float* wavelet, const int32_t* src, const int32_t* rec,
-                        const float* res, float* wgrad, bool imaging, bool illum,
-                        cudaStream_t st) {
+int fused_backward_loop(const sweep_problem* p, const Layout& L, void* ws, const float* wavelet,
+                        const int32_t* src, const int32_t* rec, const float* res, float* wgrad,
+                        bool imaging, bool illum, cudaStream_t st) {
   PhaseRange r("sweep acoustic backward");
   AcFusedArgs a = fused_args(p, L, ws, wavelet, src, rec);
   const Geom& g = a.g;
   const size_t F = sizeof(float) * (size_t)g.fstride * (size_t)g.nshot;
   cudaMemsetAsync(at<char>(ws, L.adj_lo), 0, L.adj_hi - L.adj_lo, st);
-  const int T = fused_shape(1, variant).T;
+  const int T = fused_shape(1, L.fused[1]).T;
   size_t u[2] = {0, 0}, up[2] = {0, 0};
   if (imaging) {
     cudaMemsetAsync(at<float>(ws, L.graw), 0, F, st);
@@ -727,7 +729,7 @@ int fused_backward_loop(const sweep_problem* p, const Layout& L, void* ws, int v
     a.zzo = at<float>(ws, L.zbz[o]);
     a.zxo = at<float>(ws, L.zbx[o]);
     void* tok = profile_begin(SWEEP_K_AC_BWD, st);
-    launch_ac_fused(1, variant, a, st);
+    launch_ac_fused(1, L.fused[1], a, st);
     profile_end(tok, st);
   }
   profile_end(loop, st);
@@ -738,8 +740,8 @@ int acoustic_backward_loop(const sweep_problem* p, const Layout& L, void* ws,
                            const float* wavelet, const int32_t* src, const int32_t* rec,
                            const float* res, float* wgrad, bool imaging, bool illum,
                            cudaStream_t st) {
-  if (const int v = fused_of(p, 1, imaging); v >= 0)
-    return fused_backward_loop(p, L, ws, v, wavelet, src, rec, res, wgrad, imaging, illum, st);
+  if (L.fused[1] >= 0)
+    return fused_backward_loop(p, L, ws, wavelet, src, rec, res, wgrad, imaging, illum, st);
   PhaseRange r("sweep acoustic backward");
   AcBwdLoop b;
   const int rc = b.init(p, L, ws, wavelet, src, rec, res, wgrad, imaging, illum, st);
