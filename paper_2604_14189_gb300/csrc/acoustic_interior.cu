@@ -140,14 +140,23 @@ void set_bwd_attr() {
   (void)attr;
 }
 
-// Groups of a forward CTA: two where a CTA has more than about two
-// units.  us per step with one group and with two (32-row tiles): 256 x 256 + 40,
-// 16 shots (3.5 units a CTA) 11.4, 10.2; 301 x 901 + 40, 4, 8 and 20 shots (2.5,
-// 5, 12.6) 9.1, 8.6; 12.8, 11.3; 26.8, 24.2.  Below, a larger CTA only delays the
-// CPML kernel: 301 x 901 + 40, 2 shots (1.3) 6.5, 7.8.
-int fwd_groups(long long units) {
-  const long long ctas = std::max(1LL, std::min<long long>(device_sms(), units));
-  return 4 * units >= 9 * ctas ? FWD_GROUPS : 1;
+// Groups of a forward CTA: two where a CTA has more than about two units of 32
+// rows.  us per step with one group and with two: 256 x 256 + 40, 16 shots (3.5
+// units a CTA) 11.4, 10.2; 301 x 901 + 40, 4, 8 and 20 shots (2.5, 5, 12.6) 9.1, 8.6;
+// 12.8, 11.3; 26.8, 24.2.  Below, a larger CTA only delays the CPML kernel: 301 x
+// 901 + 40, 2 shots (1.3) 6.5, 7.8.  Of 16 rows, more than 5.3 units: 301 x 901 + 40, 2,
+// 4, 5 and 8 shots (2.5, 5.05, 6.3, 10.1) 6.1, 6.8; 8.16, 8.36; 9.4, 9.0; 13.2, 11.5 (26
+// random grids: from 5.6 units on 6 to 7 % faster, from 3.3 to 5.3 from 7 % faster to
+// 2.5 % slower, below up to 18 % slower).
+int fwd_groups(const AcInFwdArgs* a, int np) {
+  long long units = 0;
+  double full = 0;  // CTAs that two groups would be worth it for
+  for (int i = 0; i < np; ++i)
+    if (a[i].units > 0) {
+      units += a[i].units;
+      full += a[i].units / (a[i].bz == IN_BZ_SMALL ? 16. / 3 : 9. / 4);
+    }
+  return full >= std::max(1LL, std::min<long long>(device_sms(), units)) ? FWD_GROUPS : 1;
 }
 
 void launch_ac_in_fwd(const AcInFwdArgs& a, cudaStream_t st) {
@@ -158,7 +167,7 @@ void launch_ac_in_fwd(const AcInFwdArgs& a, cudaStream_t st) {
   StepBatch<AcInFwdArgs, 1> m;
   m.p[0] = a;
   void* tok = profile_begin(SWEEP_K_AC_FWD_IN, st);
-  const int ng = fwd_groups(a.units);
+  const int ng = fwd_groups(&a, 1);
   launch_dependent(ng > 1 ? ac_in_fwd_kernel<1, FWD_GROUPS> : ac_in_fwd_kernel<1, 1>, dim3(grid),
                    dim3(ng * FWD_THREADS), kFwdSmem, st, m);
   profile_end(tok, st);
@@ -217,9 +226,7 @@ void launch_ac_in_fwd_batch(const AcInFwdArgs* a, int np, cudaStream_t st) {
   if (np <= 0) return;
   if (np > kStepBatch) return;  // the caller splits larger groups
   set_fwd_attr<kStepBatch>();
-  long long units = 0;
-  for (int i = 0; i < np; ++i) units += std::max(a[i].units, 0);
-  const int ng = fwd_groups(units);
+  const int ng = fwd_groups(a, np);
   launch_in_batch(ng > 1 ? ac_in_fwd_kernel<kStepBatch, FWD_GROUPS> : ac_in_fwd_kernel<kStepBatch, 1>,
                   a, np, ng * FWD_THREADS, kFwdSmem, st);
 }
