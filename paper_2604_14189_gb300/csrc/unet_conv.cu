@@ -373,7 +373,6 @@ __global__ void __launch_bounds__(kConvThreads)
   if (a.late) grid_dep_wait();
 }
 
-constexpr int kWgMaxUnits = 3;  // of a CTA
 constexpr int kWgMaxStages = 16;
 
 // Bytes of a staged chunk of kc channels: ph rows of q pw + 2 pixels, in whole
@@ -381,18 +380,6 @@ constexpr int kWgMaxStages = 16;
 __host__ __device__ inline uint32_t wg_chunk_bytes(const WgradPlan& P) {
   return (uint32_t)(P.ph * (P.q * P.pw + 2) * 2 * P.kc + 1023) / 1024 * 1024;
 }
-// Rows of strips that a set stages (ky from its first unit's to its last's).
-__host__ __device__ inline int wg_rows(const WgradPlan& P, const WgradSet& w) {
-  const int c = wgrad_chunks(P, w.block);
-  const WgradUnit l = wgrad_unit(P, c, w.u1 - 1);
-  int hi = l.ky + l.down;
-  for (int u = w.u0; u < w.u1; ++u) {
-    const WgradUnit n = wgrad_unit(P, c, u);
-    hi = n.ky + n.down > hi ? n.ky + n.down : hi;
-  }
-  return hi - wgrad_unit(P, c, w.u0).ky + 1;
-}
-
 __global__ void __launch_bounds__(kConvThreads, 2)
     wgrad_kernel(const __grid_constant__ WgradArgs a) {
   __shared__ __align__(8) uint64_t full[kWgMaxStages];
@@ -406,13 +393,15 @@ __global__ void __launch_bounds__(kConvThreads, 2)
   const uint32_t base_u = (raw_u + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (base_u - raw_u);
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  const uint32_t ncols = tmem_cols(P.per * a.cout);
+  const uint32_t ncols = tmem_cols(a.cout);
 
-  // this CTA's set (input channel block, units) and its strips
-  const int split = blockIdx.x / P.sets, set = blockIdx.x - split * P.sets;
-  const WgradSet w = wgrad_set(P, set);
-  const int chunks = wgrad_chunks(P, w.block), nu = w.u1 - w.u0, rows = wg_rows(P, w);
-  const int ky0 = wgrad_unit(P, chunks, w.u0).ky;
+  // this CTA's unit (of an input channel block) and its strips
+  const int split = blockIdx.x / P.units;
+  int u;
+  const int block = wgrad_block(P, blockIdx.x - split * P.units, &u);
+  const int chunks = wgrad_chunks(P, block);
+  const WgradUnit unit = wgrad_unit(P, chunks, u);
+  const int rows = 1 + unit.down;  // of strips
   const uint32_t CS = wg_chunk_bytes(P), DS = (uint32_t)(P.q * kWgPix * 2 * P.kb);
   const uint32_t in_bytes = (uint32_t)(rows * chunks) * CS;
   const uint32_t dy_bytes = (uint32_t)(P.q * kWgPix * 2 * a.cout);
@@ -460,7 +449,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
         for (int r = 0; r < rows; ++r)
           for (int c = 0; c < chunks; ++c)
             tma_load_4d(st + (size_t)(r * chunks + c) * CS, &a.tin, &full[s],
-                        (w.block * P.cpb + c) * P.kc, P.pw * tx - 1, P.ph * ty + ky0 + r - 1, b);
+                        (block * P.cpb + c) * P.kc, P.pw * tx - 1, P.ph * ty + unit.ky + r - 1, b);
         for (int q = 0; q < a.cout / P.kb; ++q)
           tma_load_4d(st + in_bytes + (size_t)q * DS, &a.tdy, &full[s], q * P.kb, P.pw * tx,
                       P.ph * ty, b);
@@ -487,14 +476,9 @@ __global__ void __launch_bounds__(kConvThreads, 2)
     const uint32_t la = 2u * P.kc, lb = 2u * P.kb;  // bytes of a staged pixel
     const uint64_t b0 = smem_desc(base_u + in_bytes, DS, 8u * lb,
                                   P.kb == 64 ? kSwizzle128 : kSwizzle64);
-    uint64_t a0[kWgMaxUnits];
-#pragma unroll
-    for (int u = 0; u < kWgMaxUnits; ++u) {
-      const WgradUnit n = wgrad_unit(P, chunks, min(w.u0 + u, w.u1 - 1));
-      a0[u] = smem_desc(base_u + (uint32_t)((n.ky - ky0) * chunks) * CS + (uint32_t)n.kx * la,
-                        chunks > 1 || n.down ? CS : la, 8u * la,
-                        P.kc == 64 ? kSwizzle128 : kSwizzle64);
-    }
+    const uint64_t a0 = smem_desc(base_u + (uint32_t)unit.kx * la,
+                                  chunks > 1 || unit.down ? CS : la, 8u * la,
+                                  P.kc == 64 ? kSwizzle128 : kSwizzle64);
     int s = 0, ph = 0, tx = (int)(t0 % ntx);
     uint32_t acc = 0;
     bool ok = true;
@@ -514,12 +498,9 @@ __global__ void __launch_bounds__(kConvThreads, 2)
         for (int j = 0; j < kWgPix / 16; ++j) {
           // (a strip of several rows is a stage of its own: h = 0)
           const uint32_t px = (uint32_t)(kWgPix * h + 16 * j + 2 * (16 * j / P.pw));
-          const uint64_t ao = so + (uint64_t)(px * la >> 4);
-          const uint64_t br = b0 + so + (uint64_t)((uint32_t)(kWgPix * h + 16 * j) * lb >> 4);
-#pragma unroll
-          for (int u = 0; u < kWgMaxUnits; ++u)
-            if (u < nu)
-              mma_bf16_warp(e, tmem + (uint32_t)(u * a.cout), a0[u] + ao, br, idesc, acc);
+          mma_bf16_warp(e, tmem, a0 + so + (uint64_t)(px * la >> 4),
+                        b0 + so + (uint64_t)((uint32_t)(kWgPix * h + 16 * j) * lb >> 4), idesc,
+                        acc);
           acc = 1;
         }
       }
@@ -542,14 +523,13 @@ __global__ void __launch_bounds__(kConvThreads, 2)
   tc_fence_after();
   if (!bad && warp < 4) {
     // a warp stores 32 rows of a column
-    float* out = a.partial + (size_t)blockIdx.x * P.per * a.cout * 128 + warp * 32 + lane;
-    for (int u = 0; u < nu; ++u)
-      for (int c0 = 0; c0 < a.cout; c0 += 32) {
-        float v[32];
-        tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(u * a.cout + c0), v);
+    float* out = a.partial + (size_t)blockIdx.x * a.cout * 128 + warp * 32 + lane;
+    for (int c0 = 0; c0 < a.cout; c0 += 32) {
+      float v[32];
+      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) out[((size_t)u * a.cout + c0 + i) * 128] = v[i];
-      }
+      for (int i = 0; i < 32; ++i) out[(size_t)(c0 + i) * 128] = v[i];
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -643,10 +623,8 @@ int launch_conv(ConvArgs a, cudaStream_t st) {
 }
 
 // The cut of a weight gradient.  Splits: as many as give 2 CTAs per SM with 128
-// rows of (tap, ci) each (at most kWgMaxCtas CTAs).  One unit per CTA: sets of
-// the units that share a staged row load less but leave SMs idle (8 x 256 x 256,
-// 32 -> 32: 43 us for 33; 64 -> 32: 103 for 56; others within 10 %).  partial:
-// floats of the partial sums.
+// rows of (tap, ci) each (at most kWgMaxCtas CTAs).  partial: floats of the
+// partial sums.
 WgradPlan wgrad_plan(int B, int H, int W, int cin, int cout, size_t* partial) {
   WgradPlan P{};
   P.kc = cin % 64 == 0 ? 64 : 32;
@@ -657,27 +635,28 @@ WgradPlan wgrad_plan(int B, int H, int W, int cin, int cout, size_t* partial) {
   P.pw = std::min(W, kWgPix);
   P.ph = kWgPix / P.pw;
   P.q = W >= 2 * kWgPix ? 2 : 1;  // (1 for all: 46 us for 33, 88 for 56, as above)
-  P.per = 1;
-  P.sets = (P.blocks - 1) * wgrad_block_sets(P, 0) + wgrad_block_sets(P, P.blocks - 1);
+  P.units = (P.blocks - 1) * wgrad_units(P, 0) + wgrad_units(P, P.blocks - 1);
   const long long T = (long long)B * (H / P.ph) * (W / P.pw);
   const int mtiles = (9 * cin + 127) / 128;
   P.splits = std::max(1, std::min(2 * device_sms(), kWgMaxCtas) / mtiles);
   P.splits = (int)std::max(1LL, std::min<long long>(P.splits, T));
-  size_t staged = 0;  // most of a set's
-  for (int i = 0; i < P.sets; ++i) {
-    const WgradSet w = wgrad_set(P, i);
-    staged = std::max(staged, (size_t)wg_rows(P, w) * wgrad_chunks(P, w.block) * wg_chunk_bytes(P));
+  size_t staged = 0;  // most of a unit's
+  for (int i = 0; i < P.units; ++i) {
+    int u;
+    const int chunks = wgrad_chunks(P, wgrad_block(P, i, &u));
+    staged = std::max(staged, (size_t)(1 + wgrad_unit(P, chunks, u).down) * chunks *
+                                  wg_chunk_bytes(P));
   }
   const size_t stage = staged + (size_t)P.q * kWgPix * 2 * cout;
   // (the unused runs of a short block's units read past the last stage)
   const int last = wgrad_chunks(P, P.blocks - 1);
   const size_t slack = 1024 + (last > 1 ? (size_t)(P.cpb - last) * wg_chunk_bytes(P) : 0);
-  const int cols = (int)tmem_cols(P.per * cout);
+  const int cols = (int)tmem_cols(cout);
   const int res = cols <= 256 && slack + 2 * stage <= kWgHalf ? 2 : 1;
   const size_t most = res == 2 ? kWgHalf : kWgMaxSmem;
   P.ring = (int)std::min(most - slack, kWgMaxStages * stage);
   P.smem = std::max(slack + P.ring, kSmemPerSm / (512 / cols + 1) + 1);
-  if (partial) *partial = (size_t)P.splits * P.sets * P.per * cout * 128;
+  if (partial) *partial = (size_t)P.splits * P.units * cout * 128;
   return P;
 }
 
@@ -687,7 +666,7 @@ void launch_wgrad(const WgradArgs& a, cudaStream_t st) {
     cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgMaxSmem);
   });
   const WgradPlan& P = a.plan;
-  launch_dependent(wgrad_kernel, dim3(P.splits * P.sets), dim3(kConvThreads), P.smem, st, a);
+  launch_dependent(wgrad_kernel, dim3(P.splits * P.units), dim3(kConvThreads), P.smem, st, a);
   note_launches(1);
 }
 

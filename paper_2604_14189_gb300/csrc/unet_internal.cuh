@@ -65,13 +65,15 @@ struct ConvArgs {
 //   one chunk of 64 (5 units): two taps: a pixel apart (kx = 0, 1) or a row
 //   apart (kx = 2);
 //   one chunk of 32 (3 units): unit = ky, runs a pixel apart (kx = 0, 1, 2).
-// A set is up to `per` units of a block; a CTA does one set of one split.
+// A CTA does one unit of one split.  (Several units that share a staged row load
+// less but leave SMs idle: 8 x 256 x 256, 32 -> 32 channels 43 us for 33, 64 -> 32
+// 103 for 56; other layers within 10 %.)
 constexpr int kWgPix = 64;  // pixels of a strip
 struct WgradPlan {
   int kc, nchunks, cpb, blocks;  // input channels
   int kb;                        // output channels per staged box
   int pw, ph, q;                 // columns and rows of a strip, strips of a stage
-  int per, sets, splits;
+  int units, splits;             // units of all blocks
   int ring;      // bytes of a CTA's stages
   size_t smem;
 };
@@ -79,23 +81,15 @@ __host__ __device__ inline int wgrad_chunks(const WgradPlan& P, int block) {
   const int n = P.nchunks - block * P.cpb;
   return n < P.cpb ? n : P.cpb;
 }
-__host__ __device__ inline int wgrad_units(const WgradPlan& P, int chunks) {
-  return chunks > 1 ? 9 : P.kc == 64 ? 5 : 3;
+__host__ __device__ inline int wgrad_units(const WgradPlan& P, int block) {
+  return wgrad_chunks(P, block) > 1 ? 9 : P.kc == 64 ? 5 : 3;
 }
-__host__ __device__ inline int wgrad_block_sets(const WgradPlan& P, int block) {
-  return (wgrad_units(P, wgrad_chunks(P, block)) + P.per - 1) / P.per;
-}
-struct WgradSet {
-  int block, u0, u1;
-};
-__host__ __device__ inline WgradSet wgrad_set(const WgradPlan& P, int set) {
-  WgradSet w;  // every block but the last has as many sets as the first
-  const int f = wgrad_block_sets(P, 0);
-  w.block = set / f < P.blocks - 1 ? set / f : P.blocks - 1;
-  w.u0 = (set - w.block * f) * P.per;
-  const int U = wgrad_units(P, wgrad_chunks(P, w.block));
-  w.u1 = w.u0 + P.per < U ? w.u0 + P.per : U;
-  return w;
+// Block of unit i of all, whose number in it is *u.
+__host__ __device__ inline int wgrad_block(const WgradPlan& P, int i, int* u) {
+  const int f = wgrad_units(P, 0);  // every block but the last has as many as the first
+  const int block = i / f < P.blocks - 1 ? i / f : P.blocks - 1;
+  *u = i - block * f;
+  return block;
 }
 // Tap of a unit's run 0, and whether run 1 is the tap a row below (else it is
 // the next pixel's or, with several chunks, the next chunk's).
@@ -127,7 +121,7 @@ struct WgradArgs {
   WgradPlan plan;
   int B, H, W;
   int cin, cout;
-  float* partial;    // [split][set][per][cout][128]
+  float* partial;    // [split][unit][cout][128]
   int* status;
 };
 

@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(512) bias_grad_kernel(const bf16* __restrict__
   }
 }
 
-// dW[co][tap][ci] = sum_s of its partial sums.  A column (set, unit, co) has 128
+// dW[co][tap][ci] = sum_s of its partial sums.  A column (unit, co) has 128
 // rows, four per lane.  The order is fixed: eight sums of the splits s = w,
 // w + 8, ... (each as its even and odd terms), added in turn; a warp does all
 // eight (G = 1) or, of many splits, one (G = 8).  The blocks past those sum the
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const __grid_constant
   grid_dep_trigger();
   const WgradPlan& P = a.plan;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int blocks = P.sets * P.per * a.cout * G / 8;
+  const int blocks = P.units * a.cout * G / 8;
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
   if ((int)blockIdx.x >= blocks) {
     const int c = ((int)blockIdx.x - blocks) * 32 + lane;
@@ -325,13 +325,11 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const __grid_constant
     return;
   }
   const int col = G == 8 ? blockIdx.x : blockIdx.x * 8 + w;
-  const int n = col % a.cout, q = col / a.cout;
-  const int u = q % P.per, set = q / P.per;
-  const WgradSet ws = wgrad_set(P, set);
-  if (G == 8 && ws.u0 + u >= ws.u1) return;
-  const size_t stride = (size_t)P.sets * P.per * a.cout * 32;
-  const float4* p = reinterpret_cast<const float4*>(a.partial) +
-                    ((size_t)(set * P.per + u) * a.cout + n) * 32 + lane;
+  const int n = col % a.cout;
+  int u;
+  const int block = wgrad_block(P, col / a.cout, &u);
+  const size_t stride = (size_t)P.units * a.cout * 32;
+  const float4* p = reinterpret_cast<const float4*>(a.partial) + (size_t)col * 32 + lane;
   auto sum = [&](int first) {
     float4 t0 = zero, t1 = zero;
     int s = first;
@@ -350,12 +348,12 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const __grid_constant
     __syncthreads();
     if (w) return;
     for (int k = 0; k < 8; ++k) add4(t, red[k][lane]);
-  } else if (ws.u0 + u < ws.u1) {
+  } else {
 #pragma unroll
     for (int k = 0; k < 8; ++k) add4(t, sum(k));
   }
   int tap, ci;  // (four rows lie in one run)
-  if (ws.u0 + u >= ws.u1 || !wgrad_row(P, ws.block, ws.u0 + u, 4 * lane, &tap, &ci)) return;
+  if (!wgrad_row(P, block, u, 4 * lane, &tap, &ci)) return;
   float* o = dW + ((size_t)n * 9 + tap) * a.cin + ci;
   if ((reinterpret_cast<uintptr_t>(o) & 15) == 0) {
     *reinterpret_cast<float4*>(o) = t;
@@ -444,7 +442,7 @@ void launch_bias_grad(const bf16* dy, int dy_ps, int cout, long long npix, float
 
 void launch_wgrad_reduce(const WgradArgs& a, float* dW, const float* bpart, int nb, float* db,
                          cudaStream_t st) {
-  const int cols = a.plan.sets * a.plan.per * a.cout, bias = db ? a.cout / 32 : 0;
+  const int cols = a.plan.units * a.cout, bias = db ? a.cout / 32 : 0;
   if (a.plan.splits > 32)
     launch_dependent(wgrad_reduce_kernel<8>, dim3(cols + bias), dim3(256), 0, st, a, bpart, nb, dW,
                      db);
