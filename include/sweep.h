@@ -94,7 +94,9 @@ typedef enum {
  * receivers, in receiver order, so that no two additions to a cell race.
  * Costs time (about 16 % on a 301x901 + 40 gradient).  Without it, a corner
  * cell of the border and a receiver cell inside the backward band take two
- * additions in either order, and runs agree to FP32 rounding only.  Not with
+ * additions in either order, and runs agree to FP32 rounding only.  (Small
+ * problems, whose kernels take several steps a launch, add a corner's terms in
+ * one order, x then z; only receivers that share a cell are added in any.)  Not with
  * SWEEP_F_ONE_LAUNCH (SWEEP_EUNSUPPORTED); a batched call's problems must
  * all set it or all clear it (else SWEEP_EINVAL).  Ignored for elastic
  * physics (its kernels have one writer per cell already). */

@@ -63,6 +63,9 @@ Variant bwd_variant() {
 //             2 steps, 32 x 32, one: 5.0 (141 x 187)
 //             1 step, 16 x 32, three: 5.8 | 5.7 | 8.6 | 9.3
 //             1 step, 32 x 32, two: 6.6 | 6.8 | 6.6 | 9.6
+// (The register limits that let these CTAs share an SM cost spills: forward, three
+// CTAs of 24 x 24, 136 bytes at 80 registers, the others 12 to 24 at 128; backward,
+// 32 x 32, 44 and 32 bytes at 128, the other two none.)
 // Past one wave the per-step kernels, which pipeline their loads, are as fast
 // or faster: 301 x 901 + 40 with 20 shots takes them 26.6 us forward against
 // 61.  A second wave of the last forward variant pays where the forward saves
